@@ -760,7 +760,7 @@ def run_ours(args):
     w = 4 if precision == "mixed" else 8
     E, S = info["sell_entries"], (n + 31) // 32
     kern = {  # algorithmic bytes per launch: values + columns + slice headers + vectors
-        "spmv_mech": ("k_cg_spmv<B=9> (3x3-block SELL SpMV + p.q)", E * (9 * w + 4) + S * 12 + 6 * n * w),
+        "spmv_mech": ("k_cg_spmv<B=6> (symmetric 3x3-block SELL SpMV + p.q)", E * (6 * w + 4) + S * 12 + 6 * n * w),
         "rhs_ms": ("k_fdiv (b^ms = F^ms m)", E * (3 * w + 4) + S * 12 + 3 * n * w + n * w),
         "grad_ms": ("k_fgrad (h~_d = -grad U)", E * (3 * w + 4) + S * 12 + n * w + 8 * n + 3 * n * w),
         "rhs_mech": ("k_gdiv (b^mech = F^mech E0)", E * (3 * w + 4) + S * 12 + 6 * n * w + 3 * n * w),

@@ -184,7 +184,12 @@ class Engine final : public EngineBase {
     ST(upload(&M_, ops.M));
     ST(upload(&F_, ops.F));
     ST(upload(&G_, ops.G));
-    ST(upload(&Kmech_, ops.Kmech));
+    {
+      // symmetric blocks (every mesh whose periodic faces match): 6 of 9 values
+      std::vector<double> k6;
+      kb_ = host_symmetric_blocks(hs, ops.Kmech, &k6) ? 6 : 9;
+      ST(upload(&Kmech_, kb_ == 6 ? k6 : ops.Kmech));
+    }
     // inverse diagonals of M + eps K and M + alpha eps K (Jacobi preconditioner of the GSPM
     // solves): a row's diagonal is the sum of its entries in its own column (SELL padding
     // entries point at the row itself and hold 0)
@@ -347,7 +352,7 @@ class Engine final : public EngineBase {
                             float* ms) -> int {
       CK(cudaMemcpyAsync(st, hs.data(), nseg_ * sizeof(CGState), cudaMemcpyHostToDevice,
                          L_.stream));
-      const int64_t ld = B == 9 ? 3 * n_ : (nr == 1 ? n_ : ld_);
+      const int64_t ld = B != 1 ? 3 * n_ : (nr == 1 ? n_ : ld_);
       CK(launch_cg_spmv<T>(L_, A_, SG_, val, B, nr, ld, tin_, tout_, st, red_, var, pin, diff));
       CK(cudaEventRecord(e0, L_.stream));
       for (int k = 0; k < 5; ++k)
@@ -361,7 +366,7 @@ class Engine final : public EngineBase {
     float best_b = 1e30f, best_s = 1e30f, best_g = 1e30f;
     for (int v = 0; v < kSpmvVariants; ++v) {
       float t = 0.f;
-      ST(time_variant(Kmech_, 9, 1, 1, pinned, v, &t));
+      ST(time_variant(Kmech_, kb_, 1, 1, pinned, v, &t));
       tune_ms_block_[v] = t;
       if (t < best_b) { best_b = t; var_block_ = v; }
       ST(time_variant(Kms_, 1, 1, 1, pinned, v, &t));
@@ -546,7 +551,7 @@ class Engine final : public EngineBase {
     // a6 b^mech = F^mech E0, a7 CG on pinned K^mech, x0 per the initial-guess mode
     TK(GSPM_KCLASS_RHS_MECH, launch_gdiv<T>(L_, A_, SG_, G_, sig0_, b_, pinned_));
     ST(mech_initial_guess(m_, x0_mode_));
-    ST(solve_system(kSlotMech, Kmech_, 9, b_, u_, ulo_, opt_.rtol_mech, &si->imech));
+    ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, opt_.rtol_mech, &si->imech));
     // a8 strain E = E_bar + sym grad u
     TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     // a9 h(m^n)
@@ -582,7 +587,7 @@ class Engine final : public EngineBase {
       TK(GSPM_KCLASS_POINTWISE, launch_e0<T>(L_, n, ms_, ld, mag_, D, E0_, sig0_));
       TK(GSPM_KCLASS_POINTWISE, launch_wsum<T>(L_, SG_, 6, E0_, ld, 1, nullptr, w_, ebar(), eext(), red_));
       TK(GSPM_KCLASS_RHS_MECH, launch_gdiv<T>(L_, A_, SG_, G_, sig0_, b_, pinned_));
-      ST(solve_system(kSlotMech, Kmech_, 9, b_, u_, ulo_, opt_.rtol_mech, &si->imech2));
+      ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, opt_.rtol_mech, &si->imech2));
       TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     }
     TK(GSPM_KCLASS_POINTWISE, launch_hfield<T>(L_, n, SG_, ms_, hd_, E_, ld, mbar_s(), hz(), mag_, D, 1, P_.alpha * P_.dtau, nullptr, x_));
@@ -848,7 +853,7 @@ class Engine final : public EngineBase {
     TK(GSPM_KCLASS_POINTWISE, launch_wsum<T>(L_, SG_, 6, E0_, ld, 1, nullptr, w_, ebar(), eext(), red_));
     TK(GSPM_KCLASS_RHS_MECH, launch_gdiv<T>(L_, A_, SG_, G_, sig0_, b_, pinned_));
     std::vector<SolveInfo> info;
-    ST(solve_system(kSlotMech, Kmech_, 9, b_, u_, ulo_, rtol > 0 ? rtol : opt_.rtol_mech, &info));
+    ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, rtol > 0 ? rtol : opt_.rtol_mech, &info));
     TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     if (u) ST(export_field(u_, 1, 3, 3, u, where, ulo_));
     CK(cudaStreamSynchronize(L_.stream));
@@ -901,7 +906,7 @@ class Engine final : public EngineBase {
       case GSPM_OP_K_MECH:
         ST(import_field(x, where, 3, tin_, 1, 3, nullptr));
         ST(pin_hide(3));
-        CK(launch_spmv<T>(L_, A_, Kmech_, 9, tin_, tout_, var_block_, 1));
+        CK(launch_spmv<T>(L_, A_, Kmech_, kb_, tin_, tout_, var_block_, 1));
         ST(pin_restore(3));
         ST(export_field(tout_, 1, 3, 3, y, where));
         break;
@@ -1264,7 +1269,7 @@ class Engine final : public EngineBase {
     return GSPM_OK;
   }
 
-  // K x = b for one K^ms (B = 1) or K^mech (B = 9) solve.  Mixed precision: iterative
+  // K x = b for one K^ms (B = 1) or K^mech (B = kb_) solve.  Mixed precision: iterative
   // refinement (Wilkinson's scheme with the working-precision solver run in FP32): a first FP32
   // CG solve to kRtolInner leaves x; a second CG restarts from x, its initial residual b - K x
   // formed to twice the working precision (k_cg_init), and accumulates the correction in the
@@ -1275,7 +1280,7 @@ class Engine final : public EngineBase {
   // much smaller dx.  FP64 (xlo == NULL): one solve.
   int solve_system(int slot, const T* val, int B, const T* b, T* x, T* xlo, double rtol,
                    std::vector<SolveInfo>* info) {
-    const int epr = B == 9 ? 3 : 1;
+    const int epr = B == 1 ? 1 : 3;
     const int slot2 = slot == kSlotMs ? kSlotMs2 : kSlotMech2;
     if (!xlo) {
       ST(solve_general(slot, val, B, b, x, x, rtol, info));
@@ -1297,19 +1302,19 @@ class Engine final : public EngineBase {
       }
     }
     if (tres_on_)
-      TK(GSPM_KCLASS_CG_INIT, launch_true_res<T>(L_, A_, SG_, val, B, b, x, xlo, red_, tres_ + (B == 9 ? 2 * nseg_ : 0)));
+      TK(GSPM_KCLASS_CG_INIT, launch_true_res<T>(L_, A_, SG_, val, B, b, x, xlo, red_, tres_ + (B == 1 ? 0 : 2 * nseg_)));
     return GSPM_OK;
   }
 
-  // CG for K x = b (B = 1 scalar K^ms, B = 9 block K^mech), pinned or singular form, started from
+  // CG for K x = b (B = 1 scalar K^ms, B = kb_ block K^mech), pinned or singular form, started from
   // x0 (read only) with the iterates accumulated into x: x == x0 is the plain solve; x != x0
   // (zero on entry) is the correction solve of solve_system, whose solution is x0 + x
   int solve_general(int slot, const T* val, int B, const T* b, const T* x0, T* x, double rtol,
                     std::vector<SolveInfo>* info) {
-    Trace trace(B == 9 ? "cg_mech" : "cg_ms");
+    Trace trace(B == 1 ? "cg_ms" : "cg_mech");
     CGState* st = cg_ + (int64_t)slot * nseg_;
     int* na = nactive_ + slot;
-    const int epr = B == 9 ? 3 : 1;
+    const int epr = B == 1 ? 1 : 3;
     const int64_t len = epr * n_;
     double* bmean = proj_;
     double* xpin = proj_ + 3 * nseg_;
@@ -1344,7 +1349,7 @@ class Engine final : public EngineBase {
     // singular system: p0 projected off the constants
     if (!pinned_) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
     auto iter = [&]() -> int {
-      TK(B == 9 ? GSPM_KCLASS_SPMV_MECH : GSPM_KCLASS_SPMV_MS, launch_cg_spmv<T>(L_, A_, SG_, val, B, 1, len, p_, q_, st, red_, B == 9 ? var_block_ : var_scalar_, pinned_, 1));
+      TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_spmv<T>(L_, A_, SG_, val, B, 1, len, p_, q_, st, red_, B == 1 ? var_scalar_ : var_block_, pinned_, 1));
       TK(GSPM_KCLASS_CG_VEC, launch_cg_update<T>(L_, SG_, epr, 1, len, x, r_, p_, q_, st, na, red_));
       if (pc) {
         // z into q (free after the update), then p = z + beta p
@@ -1356,7 +1361,7 @@ class Engine final : public EngineBase {
       return GSPM_OK;
     };
     if (capturing_)
-      ST(cg_graph_loop(slot, iter, B == 9 ? 1 : 0, pc ? 7 : 3));
+      ST(cg_graph_loop(slot, iter, B == 1 ? 0 : 1, pc ? 7 : 3));
     else
       ST(cg_loop(slot, iter, info));
     // singular system: move the solution to the pinned one (zero at the pinned node)
@@ -1791,6 +1796,7 @@ class Engine final : public EngineBase {
   gspm_options opt_;
   Launch L_;
   DevMem mem_;
+  int kb_ = 9;  // stored values per K^mech block: 6 (symmetric) or 9
   int64_t n_ = 0, ld_ = 0, nslices_ = 0, entries_ = 0, nmag_ = 0, nodes_ = 0;
   int nseg_ = 1, nitems_ = 0, item_slices_ = 1;
   DSeg SG_{};

@@ -714,6 +714,31 @@ void host_assemble(const HostMesh& hm, const HostSell& s, const Params& p, HostO
   }
 }
 
+bool host_symmetric_blocks(const HostSell& s, const std::vector<double>& k9,
+                           std::vector<double>* k6) {
+  static const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
+  k6->assign(6 * s.entries, 0.0);
+  int bad = 0;
+#pragma omp parallel for schedule(static) reduction(| : bad)
+  for (int64_t sl = 0; sl < s.nslices; ++sl)
+    for (int lane = 0; lane < kSell; ++lane) {
+      double big = 0.0, off = 0.0;
+      for (int k = 0; k < s.slen[sl]; ++k) {
+        const int64_t e = s.sptr[sl] + (int64_t)k * kSell;
+        const double* a = &k9[9 * e + lane];
+        for (int q = 0; q < 9; ++q) big = std::max(big, std::fabs(a[q * kSell]));
+        for (int q = 0; q < 6; ++q) {
+          const double u = a[(3 * ia[q] + ib[q]) * kSell], v = a[(3 * ib[q] + ia[q]) * kSell];
+          off = std::max(off, std::fabs(u - v));
+          (*k6)[6 * e + q * kSell + lane] = u + 0.5 * (v - u);
+        }
+      }
+      if (!(off <= 1e-13 * big)) bad |= 1;
+    }
+  if (bad) k6->clear();
+  return !bad;
+}
+
 void host_batch_build(std::vector<HostMesh>& hm, std::vector<HostSell>& hs,
                       std::vector<HostOps>& ops, HostBatch* b) {
   const int S = (int)hm.size();

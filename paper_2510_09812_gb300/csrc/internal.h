@@ -99,6 +99,14 @@ struct HostOps {
 };
 void host_assemble(const HostMesh& hm, const HostSell& s, const Params& p, HostOps* ops);
 
+// Upper triangles (00, 01, 02, 11, 12, 22) of the 3x3 blocks of a SELL matrix with nine values per
+// entry, as a matrix with six.  False (k6 empty) unless every block is symmetric: |A_ab - A_ba| at
+// most 1e-13 of the largest value of its row (blocks summed over some 24 elements in FP64 differ
+// by a few 1e-16; a periodic wrap that identifies nodes which do not match, within a large
+// wrap_tol, leaves larger differences).  Stored is the mean of A_ab and A_ba.
+bool host_symmetric_blocks(const HostSell& s, const std::vector<double>& k9,
+                           std::vector<double>* k6);
+
 // Two-level preconditioner of the K^ms and K^mech solves: plain aggregation P (node i -> its
 // aggregate, the same for every displacement component), coarse operators P^T K P, their
 // inverses after the null space (the constants of each component) is shifted by

@@ -17,398 +17,12 @@
 #include <type_traits>
 #include <unordered_map>
 
+#include "device.cuh"
 #include "kernels.cuh"
 
 namespace gspm {
 
 namespace {
-
-constexpr unsigned kFull = 0xffffffffu;
-
-__device__ __forceinline__ double warp_sum(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-  return x;
-}
-
-// Compensated summation (Kahan): s + c carries the running sum with the low-order part lost by
-// each add kept in c (subtracted at the end: total = s - c)
-template <typename T>
-__device__ __forceinline__ void kahan_add(T& s, T& c, T x) {
-  const T y = x - c;
-  const T t = s + y;
-  c = (t - s) - y;
-  s = t;
-}
-
-__device__ __forceinline__ int64_t gtid() { return (int64_t)blockIdx.x * blockDim.x + threadIdx.x; }
-__device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * blockDim.x; }
-
-// Programmatic dependent launch (the CG loop kernels): a kernel launched with
-// launch_pdl first waits until the previous kernel of the stream has completed and its memory
-// is visible, then lets the next kernel be scheduled (its blocks wait the same way), so
-// launch latency overlaps the running kernel.  Outside such a launch both are no-ops.
-__device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-// The last item of `seg` to arrive (its block partials already in red.partial[item]) sums the
-// segment's item partials in item order and returns true (totals in res[0..NC), valid in every
-// thread of that block).
-template <int NC>
-__device__ __forceinline__ bool seg_arrive(int item, int seg, const DSeg& G, const ItemList& IL,
-                                           const Red& red, double* res) {
-  __shared__ double sm[NC][32];
-  __shared__ int am_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned t = atomicAdd(G.counter + seg, 1u);
-    am_last = (t == (unsigned)IL.seg_nitems[seg] - 1u);
-  }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  const int i0 = IL.seg_item0[seg], ni = IL.seg_nitems[seg];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < ni; b += blockDim.x)
-      acc += __ldcg(red.partial + (int64_t)(i0 + b) * kRedComp + c);
-    acc = warp_sum(acc);
-    if (lane == 0) sm[c][warp] = acc;
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const double x = warp_sum(lane < nw ? sm[c][lane] : 0.0);
-      if (lane == 0) res[c] = x;
-    }
-  }
-  if (threadIdx.x == 0) G.counter[seg] = 0u;
-  __syncthreads();
-  return true;
-}
-
-// Block reduction of NC values into partial[item] (FP64 tree), then seg_arrive.
-template <int NC>
-__device__ __forceinline__ bool seg_reduce(double (&v)[NC], int item, int seg, const DSeg& G,
-                                           const ItemList& IL, const Red& red, double* res) {
-  __shared__ double sm[NC][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    const double x = warp_sum(v[c]);
-    if (lane == 0) sm[c][warp] = x;
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const double x = warp_sum(lane < nw ? sm[c][lane] : 0.0);
-      if (lane == 0) red.partial[(int64_t)item * kRedComp + c] = x;
-    }
-  }
-  return seg_arrive<NC>(item, seg, G, IL, red, res);
-}
-
-// Double-float addition (h, l) += (bh, bl): Knuth's TwoSum of the high parts, the low parts
-// added to its error term, renormalised (the _rn intrinsics keep the compiler from contracting
-// or reassociating the steps)
-__device__ __forceinline__ void df_add(float& h, float& l, float bh, float bl) {
-  const float s = __fadd_rn(h, bh);
-  const float z = __fsub_rn(s, h);
-  float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, z)), __fsub_rn(bh, z));
-  e = __fadd_rn(e, __fadd_rn(l, bl));
-  h = __fadd_rn(s, e);
-  l = __fsub_rn(e, __fsub_rn(h, s));
-}
-
-// seg_reduce of per-thread values given as unevaluated sums hi + lo in T.  T = float: the warp
-// and block trees run in double-float arithmetic (FP32 operations, about 44 significant bits;
-// an FP64 instruction costs ~64 FP32 ones on this part and the FP64 trees dominated the short
-// CG vector kernels), one FP64 conversion per block and value.  T = double: seg_reduce.
-template <typename T, int NC>
-__device__ __forceinline__ bool seg_reduce_hl(const T (&hi)[NC], const T (&lo)[NC], int item,
-                                              int seg, const DSeg& G, const ItemList& IL,
-                                              const Red& red, double* res) {
-  if constexpr (std::is_same<T, double>::value) {
-    double v[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) v[c] = hi[c] + lo[c];
-    return seg_reduce<NC>(v, item, seg, G, IL, red, res);
-  } else {
-    __shared__ float smh[NC][32], sml[NC][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      float h = hi[c], l = lo[c];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float bh = __shfl_down_sync(kFull, h, o), bl = __shfl_down_sync(kFull, l, o);
-        df_add(h, l, bh, bl);
-      }
-      if (lane == 0) {
-        smh[c][warp] = h;
-        sml[c][warp] = l;
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        float h = lane < nw ? smh[c][lane] : 0.f, l = lane < nw ? sml[c][lane] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float bh = __shfl_down_sync(kFull, h, o), bl = __shfl_down_sync(kFull, l, o);
-          df_add(h, l, bh, bl);
-        }
-        if (lane == 0) red.partial[(int64_t)item * kRedComp + c] = (double)h + (double)l;
-      }
-    }
-    return seg_arrive<NC>(item, seg, G, IL, red, res);
-  }
-}
-
-// The difference forms sum_j A_ij (x_j - x_i) of the zero-row-sum operators (K^ms, K^mech, F^ms,
-// G) are used in FP32, where they keep smooth fields from cancelling; in FP64 the plain products
-// are accurate enough and each extra subtraction costs FP64 issue slots.
-template <typename T>
-constexpr int kDiff = std::is_same<T, float>::value ? 1 : 0;
-
-__device__ __forceinline__ bool row_valid(const DSeg& G, int seg, int64_t row) {
-  return row - G.seg_row0[seg] < G.seg_nrow[seg];
-}
-
-// y_r(row) = sum_k A(row, k) x_r(col(row, k)) for one row of a scalar SELL matrix, neighbours
-// k = k0, k0 + kstep, ...  diff != 0 (an operator whose rows sum to zero: K^ms, K^mech): formed as
-// sum_k A(row, k) (x_r(col) - x_r(row)), equal in exact arithmetic; a smooth x then does not
-// cancel in the sum, and the FP32 rounding of the values cannot make the operator act on the
-// constants (its rows' rounded sums no longer enter).
-template <typename V, typename X, typename Acc, int NR, int VAR = 0>
-__device__ __forceinline__ void sell_scalar_row(const DSell& A, const V* __restrict__ val,
-                                                int64_t s, int lane, const X* __restrict__ x,
-                                                int64_t ld, const int (&skip)[NR],
-                                                Acc (&acc)[NR], int k0 = 0, int kstep = 1,
-                                                int diff = 0) {
-  const int64_t base = A.sptr[s];
-  const int len = A.slen[s];
-  const int32_t* cp = A.col + base + lane;
-  const V* vp = val + base + lane;
-  const int64_t row = s * 32 + lane;
-  X xi[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) {
-    acc[r] = Acc(0);
-    xi[r] = diff && row < A.n ? x[r * ld + row] : X(0);
-  }
-  if (VAR == 1 || VAR == 3) {
-    // eight neighbours per round: their columns and values first, then the gathers, then the
-    // FMAs (more loads in flight per thread).  Past the row's end the round re-reads entry kb
-    // (kb < len), so every load is unconditional and inside the slice, with weight 0.
-    for (int kb = k0; kb < len; kb += 8 * kstep) {
-      int j[8];
-      V w[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = kb + u * kstep;
-        const int kc = k < len ? k : kb;
-        j[u] = __ldcs(cp + (int64_t)kc * 32);
-        const V wv = __ldcs(vp + (int64_t)kc * 32);
-        w[u] = k < len ? wv : V(0);
-      }
-#pragma unroll
-      for (int r = 0; r < NR; ++r)
-        if (!skip[r]) {
-          X g[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) g[u] = __ldg(x + r * ld + j[u]) - xi[r];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[r] += (Acc)w[u] * (Acc)g[u];
-        }
-    }
-    return;
-  }
-#pragma unroll 4
-  for (int k = k0; k < len; k += kstep) {
-    const int j = __ldcs(cp + (int64_t)k * 32);
-    const Acc a = (Acc)__ldcs(vp + (int64_t)k * 32);
-#pragma unroll
-    for (int r = 0; r < NR; ++r)
-      if (!skip[r]) acc[r] += a * (Acc)(__ldg(x + r * ld + j) - xi[r]);
-  }
-}
-
-// 3x3-block row: y(row, a) = sum_k sum_b A(row, k)_ab x(col, b); x, y arrays of [n][3].
-// diff != 0: sum_k A(row, k) (x(col) - x(row)), as in sell_scalar_row.
-template <typename V, typename X, typename Acc, int VAR>
-__device__ __forceinline__ void sell_block_row(const DSell& A, const V* __restrict__ val,
-                                               int64_t s, int lane, const X* __restrict__ x,
-                                               Acc (&acc)[3], int k0 = 0, int kstep = 1,
-                                               int diff = 0) {
-  const int64_t base = A.sptr[s];
-  const int len = A.slen[s];
-  const int32_t* cp = A.col + base + lane;
-  const V* vp = val + base * 9 + lane;
-  const int64_t row = s * 32 + lane;
-  const bool own = diff && row < A.n;
-  const X xi0 = own ? x[3 * row] : X(0), xi1 = own ? x[3 * row + 1] : X(0),
-          xi2 = own ? x[3 * row + 2] : X(0);
-  acc[0] = acc[1] = acc[2] = Acc(0);
-  if (VAR == 1 || VAR == 3) {
-    // five neighbours per round: all loads first, then the FMAs; past the row's end entry kb
-    // is re-read with weight 0 (unconditional loads, all inside the slice)
-    for (int kb = k0; kb < len; kb += 5 * kstep) {
-      int j[5];  // 32-bit: five fewer registers than 64-bit indices in this unrolled round
-      V w[5][9];
-#pragma unroll
-      for (int u = 0; u < 5; ++u) {
-        const int k = kb + u * kstep;
-        const bool ok = k < len;
-        const int kc = ok ? k : kb;
-        j[u] = __ldcs(cp + (int64_t)kc * 32);
-        const V* bp = vp + (int64_t)kc * 288;
-#pragma unroll
-        for (int e = 0; e < 9; ++e) {
-          const V wv = __ldcs(bp + e * 32);
-          w[u][e] = ok ? wv : V(0);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 5; ++u) {
-        const X* xj = x + 3 * (int64_t)j[u];
-        const Acc x0 = (Acc)(__ldg(xj) - xi0), x1 = (Acc)(__ldg(xj + 1) - xi1),
-                  x2 = (Acc)(__ldg(xj + 2) - xi2);
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-          acc[a] += (Acc)w[u][3 * a] * x0 + (Acc)w[u][3 * a + 1] * x1 + (Acc)w[u][3 * a + 2] * x2;
-      }
-    }
-  } else {
-#pragma unroll 2
-    for (int k = k0; k < len; k += kstep) {
-      const int64_t j = __ldcs(cp + (int64_t)k * 32);
-      const V* bp = vp + (int64_t)k * 288;
-      const Acc x0 = (Acc)(__ldg(x + 3 * j) - xi0), x1 = (Acc)(__ldg(x + 3 * j + 1) - xi1),
-                x2 = (Acc)(__ldg(x + 3 * j + 2) - xi2);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        acc[a] += (Acc)__ldcs(bp + (3 * a + 0) * 32) * x0;
-        acc[a] += (Acc)__ldcs(bp + (3 * a + 1) * 32) * x1;
-        acc[a] += (Acc)__ldcs(bp + (3 * a + 2) * 32) * x2;
-      }
-    }
-  }
-}
-
-// Compensated dot product in FP32 (Ogita, Rump and Oishi, "Accurate sum and dot product", SIAM
-// J. Sci. Comput. 26 (2005), Algorithm Dot2): each product is split exactly into p + e with an
-// FMA, the running sum kept exactly as s plus the accumulated errors c by Knuth's TwoSum, so
-// s + c is as accurate as the dot product computed in twice the working precision.  The CG
-// initial residuals b - A x (which cancel heavily with a warm start) use it instead of FP64
-// arithmetic, whose rate on this part is 1/64 of FP32's.
-struct Dot2 {
-  float s = 0.f, c = 0.f;
-  // the _rn intrinsics keep the compiler from contracting or reassociating these steps
-  __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b);
-    const float e = fmaf(a, b, -p);
-    const float t = __fadd_rn(s, p);
-    const float z = __fsub_rn(t, s);
-    const float d = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
-    c = __fadd_rn(c, __fadd_rn(d, e));
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-
-// sell_scalar_row / sell_block_row with Dot2 accumulators (FP32 operands)
-template <int NR>
-__device__ __forceinline__ void sell_scalar_row_dot2(const DSell& A, const float* __restrict__ val,
-                                                     int64_t s, int lane,
-                                                     const float* __restrict__ x, int64_t ld,
-                                                     Dot2 (&acc)[NR], int diff = 0) {
-  const int64_t base = A.sptr[s];
-  const int len = A.slen[s];
-  const int32_t* cp = A.col + base + lane;
-  const float* vp = val + base + lane;
-  const int64_t row = s * 32 + lane;
-  float xi[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) xi[r] = diff && row < A.n ? x[r * ld + row] : 0.f;
-#pragma unroll 4
-  for (int k = 0; k < len; ++k) {
-    const int j = __ldcs(cp + (int64_t)k * 32);
-    const float a = __ldcs(vp + (int64_t)k * 32);
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc[r].add(a, __fsub_rn(__ldg(x + r * ld + j), xi[r]));
-  }
-}
-__device__ __forceinline__ void sell_block_row_dot2(const DSell& A, const float* __restrict__ val,
-                                                    int64_t s, int lane,
-                                                    const float* __restrict__ x,
-                                                    Dot2 (&acc)[3], int diff = 0) {
-  const int64_t base = A.sptr[s];
-  const int len = A.slen[s];
-  const int32_t* cp = A.col + base + lane;
-  const float* vp = val + base * 9 + lane;
-  const int64_t row = s * 32 + lane;
-  const bool own = diff && row < A.n;
-  const float xi0 = own ? x[3 * row] : 0.f, xi1 = own ? x[3 * row + 1] : 0.f,
-              xi2 = own ? x[3 * row + 2] : 0.f;
-#pragma unroll 2
-  for (int k = 0; k < len; ++k) {
-    const int64_t j = __ldcs(cp + (int64_t)k * 32);
-    const float* bp = vp + (int64_t)k * 288;
-    const float x0 = __fsub_rn(__ldg(x + 3 * j), xi0), x1 = __fsub_rn(__ldg(x + 3 * j + 1), xi1),
-                x2 = __fsub_rn(__ldg(x + 3 * j + 2), xi2);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      acc[a].add(__ldcs(bp + (3 * a + 0) * 32), x0);
-      acc[a].add(__ldcs(bp + (3 * a + 1) * 32), x1);
-      acc[a].add(__ldcs(bp + (3 * a + 2) * 32), x2);
-    }
-  }
-}
-
-// Work unit of the SELL kernels for schedule VAR: one slice per warp (VAR 0, 1), or half a slice
-// per warp with two lanes per row (VAR 2).  unit_row() gives, for this lane, the slice, the SELL
-// lane of its row, and the first neighbour and stride it handles.
-template <int VAR>
-__device__ __forceinline__ void unit_row(int64_t u, int lane, int64_t& s, int& sl, int& k0,
-                                         int& kstep) {
-  if (VAR == 2) {
-    s = u >> 1;
-    sl = (int)(u & 1) * 16 + (lane & 15);
-    k0 = lane >> 4;
-    kstep = 2;
-  } else {
-    s = u;
-    sl = lane;
-    k0 = 0;
-    kstep = 1;
-  }
-}
-// minimum resident blocks per SM a schedule is compiled for (register cap)
-template <int VAR>
-constexpr int min_blocks() {
-  return VAR == 3 ? 3 : 1;
-}
-template <int VAR>
-__device__ __forceinline__ int units_per_slice() {
-  return VAR == 2 ? 2 : 1;
-}
-// combine the two partial row results of VAR 2 (lanes l and l+16); true on the lane that owns
-// the row's result
-template <int VAR, typename Acc, int N>
-__device__ __forceinline__ bool unit_combine(Acc (&acc)[N], int lane) {
-  if (VAR != 2) return true;
-#pragma unroll
-  for (int a = 0; a < N; ++a) acc[a] += __shfl_xor_sync(kFull, acc[a], 16);
-  return lane < 16;
-}
 
 // ------------------------------------------------------------------------------------------
 // volume average per segment: out[seg*nc + c] = sum_i w_i f(i, c) (+ add[c]); Sec. 2.4 with
@@ -461,7 +75,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_spmv1(DSell A, co
   }
 }
 
-template <typename T, int VAR>
+template <typename T, int B, int VAR>
 __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_spmv9(DSell A, const T* __restrict__ val,
                                                   const T* __restrict__ x, T* __restrict__ y,
                                                   int diff) {
@@ -472,7 +86,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_spmv9(DSell A, co
     int sl, k0, ks;
     unit_row<VAR>(u, lane, s, sl, k0, ks);
     T acc[3];
-    sell_block_row<T, T, T, VAR>(A, val, s, sl, x, acc, k0, ks, diff);
+    sell_block_row<B, T, T, T, VAR>(A, val, s, sl, x, acc, k0, ks, diff);
     const int64_t row = s * 32 + sl;
     if (unit_combine<VAR>(acc, lane) && row < A.n) {
       y[3 * row] = acc[0];
@@ -519,7 +133,7 @@ __device__ __forceinline__ void cg_start(CGState* st, int* nactive, int nr, cons
   if (any) atomicAdd(nactive, 1);
 }
 
-// r = b' - A x, p = r (scalar B = 1 or 3x3 block B = 9), one right-hand side, where
+// r = b' - A x, p = r (scalar B = 1, or 3x3 block B = 6 or 9), one right-hand side, where
 //   bmean != NULL: b' = b - bmean[seg] per component (the consistent singular system's
 //                  right-hand side: b projected off the constants),
 //   pinned:        b' = b with r = 0 at the segment's pinned row (the pinned system; x and b
@@ -533,7 +147,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_init(DSell A, DSeg G, ItemList IL
                                                     int max_iter, Red red,
                                                     const double* __restrict__ bmean,
                                                     int pinned, int pc) {
-  constexpr int NC = B == 9 ? 3 : 1;
+  constexpr int NC = B == 1 ? 1 : 3;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
     const int seg = IL.seg[item];
@@ -549,7 +163,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_init(DSell A, DSeg G, ItemList IL
       const bool ok = row_valid(G, seg, row);
       // A x to twice the working precision (FP64, or compensated FP32): with a good initial
       // guess b - A x cancels heavily
-      if (B == 1) {
+      if constexpr (B == 1) {
         double acc[1];
         if constexpr (std::is_same<T, float>::value) {
           Dot2 d[1];
@@ -572,10 +186,10 @@ __global__ void __launch_bounds__(kBlock) k_cg_init(DSell A, DSeg G, ItemList IL
         double acc[3];
         if constexpr (std::is_same<T, float>::value) {
           Dot2 d[3];
-          sell_block_row_dot2(A, val, s, lane, x, d, 1);
+          sell_block_row_dot2<B>(A, val, s, lane, x, d, 1);
           for (int a = 0; a < 3; ++a) acc[a] = d[a].value();
         } else {
-          sell_block_row<T, T, double, 0>(A, val, s, lane, x, acc, 0, 1, kDiff<T>);
+          sell_block_row<B, T, T, double, 0>(A, val, s, lane, x, acc, 0, 1, kDiff<T>);
         }
         if (ok) {
 #pragma unroll
@@ -674,7 +288,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_init_gs(DSell A, DSeg G, ItemList
   }
 }
 
-// True residual of a finished K^ms (B = 1) or K^mech (B = 9) solve, independent of the CG
+// True residual of a finished K^ms (B = 1) or K^mech (B = 6 or 9) solve, independent of the CG
 // recursion: per segment, over every row but the pinned one, sum (b - A x)^2 and b^2 into
 // out[2 seg] and out[2 seg + 1].  A x is accumulated in FP64 (a product of two FP32 values is
 // exact in FP64), so the result measures the solution against the operator as stored.  x is
@@ -686,7 +300,7 @@ __global__ void __launch_bounds__(kBlock) k_true_res(DSell A, DSeg G, ItemList I
                                                      const T* __restrict__ x,
                                                      const T* __restrict__ xlo, Red red,
                                                      double* out) {
-  constexpr int NC = B == 9 ? 3 : 1;
+  constexpr int NC = B == 1 ? 1 : 3;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
     const int seg = IL.seg[item];
@@ -695,7 +309,7 @@ __global__ void __launch_bounds__(kBlock) k_true_res(DSell A, DSeg G, ItemList I
     for (int64_t s = IL.sl0[item] + warp; s < IL.sl1[item]; s += kBlock / 32) {
       const int64_t row = s * 32 + lane;
       double acc[3] = {0.0, 0.0, 0.0};
-      if (B == 1) {
+      if constexpr (B == 1) {
         const int skip[1] = {0};
         double a1[1];
         sell_scalar_row<T, T, double, 1>(A, val, s, lane, x, 0, skip, a1, 0, 1, kDiff<T>);
@@ -705,10 +319,10 @@ __global__ void __launch_bounds__(kBlock) k_true_res(DSell A, DSeg G, ItemList I
           acc[0] += a1[0];
         }
       } else {
-        sell_block_row<T, T, double, 0>(A, val, s, lane, x, acc, 0, 1, kDiff<T>);
+        sell_block_row<B, T, T, double, 0>(A, val, s, lane, x, acc, 0, 1, kDiff<T>);
         if (xlo) {
           double a3[3];
-          sell_block_row<T, T, double, 0>(A, val, s, lane, xlo, a3, 0, 1, kDiff<T>);
+          sell_block_row<B, T, T, double, 0>(A, val, s, lane, xlo, a3, 0, 1, kDiff<T>);
           for (int a = 0; a < 3; ++a) acc[a] += a3[a];
         }
       }
@@ -759,7 +373,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_cg_spmv(DSell A, 
       int sl, k0, ks;
       unit_row<VAR>(u, lane, s, sl, k0, ks);
       const int64_t row = s * 32 + sl;
-      if (B == 1) {
+      if constexpr (B == 1) {
         T acc[NR];
         sell_scalar_row<T, T, T, NR, VAR>(A, val, s, sl, p, ld, skip, acc, k0, ks, DIFF);
         if (row == pin) {
@@ -776,7 +390,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_cg_spmv(DSell A, 
         }
       } else {
         T acc[3];
-        sell_block_row<T, T, T, VAR>(A, val, s, sl, p, acc, k0, ks, DIFF);
+        sell_block_row<B, T, T, T, VAR>(A, val, s, sl, p, acc, k0, ks, DIFF);
         if (row == pin) acc[0] = acc[1] = acc[2] = T(0);
         if (unit_combine<VAR>(acc, lane) && row_valid(G, seg, row)) {
           T pq = T(0);
@@ -2083,8 +1697,11 @@ static void spmv_variant(const Launch& L, const DSell& A, const T* val, int B, c
   if (B == 1) {
     auto k = k_spmv1<T, VAR>;
     k<<<GSPM_GRID(L, threads, k), kBlock, 0, L.stream>>>(A, val, x, y, diff);
+  } else if (B == 6) {
+    auto k = k_spmv9<T, 6, VAR>;
+    k<<<GSPM_GRID(L, threads, k), kBlock, 0, L.stream>>>(A, val, x, y, diff);
   } else {
-    auto k = k_spmv9<T, VAR>;
+    auto k = k_spmv9<T, 9, VAR>;
     k<<<GSPM_GRID(L, threads, k), kBlock, 0, L.stream>>>(A, val, x, y, diff);
   }
 }
@@ -2113,6 +1730,11 @@ cudaError_t launch_cg_init(const Launch& L, const DSell& A, const DSeg& G, const
     const ItemGrid ig = GSPM_IGRID(L, G, k);
     k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, r, p, st, nactive, rtol,
                                         max_iter, red, bmean, pinned, pc);
+  } else if (B == 6) {
+    auto k = k_cg_init<T, 6>;
+    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, r, p, st, nactive, rtol,
+                                        max_iter, red, bmean, pinned, pc);
   } else {
     auto k = k_cg_init<T, 9>;
     const ItemGrid ig = GSPM_IGRID(L, G, k);
@@ -2128,6 +1750,10 @@ cudaError_t launch_true_res(const Launch& L, const DSell& A, const DSeg& G, cons
   (*L.counter) += 1;
   if (B == 1) {
     auto k = k_true_res<T, 1>;
+    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, xlo, red, out);
+  } else if (B == 6) {
+    auto k = k_true_res<T, 6>;
     const ItemGrid ig = GSPM_IGRID(L, G, k);
     k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, xlo, red, out);
   } else {
@@ -2204,7 +1830,11 @@ template <typename T, int VAR>
 static cudaError_t cg_spmv_variant(const Launch& L, const DSell& A, const DSeg& G, const T* val,
                                    int B, int nr, int64_t ld, const T* p, T* q, CGState* st,
                                    Red red, int pinned, int diff) {
-  if (B == 9) {
+  if (B == 6) {
+    auto k = k_cg_spmv<T, 6, 1, VAR, kDiff<T>>;
+    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
+  } else if (B == 9) {
     auto k = k_cg_spmv<T, 9, 1, VAR, kDiff<T>>;
     const ItemGrid ig = GSPM_IGRID(L, G, k);
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);

@@ -134,7 +134,7 @@ cudaError_t launch_wsum(const Launch& L, const DSeg& G, int nc, const T* f, int6
                         const double* add, Red red);  // out[seg * nc + c]
 template <typename T>
 cudaError_t launch_spmv(const Launch& L, const DSell& A, const T* val, int B, const T* x,
-                        T* y, int variant = 0, int diff = 0);  // B = 1 scalar, B = 9 block
+                        T* y, int variant = 0, int diff = 0);  // B = 1 scalar, B = 6 or 9 block
 // (x, y AoS 3); diff != 0: the operator's rows sum to zero (K^ms, K^mech) and each row is
 // formed as sum_j A_ij (x_j - x_i)
 // CG pieces.  st and the arrival counters are per segment; nactive counts active segments.
@@ -152,7 +152,7 @@ cudaError_t launch_cg_init(const Launch& L, const DSell& A, const DSeg& G, const
                            int max_iter, Red red, const double* bmean, int pinned, int pc);
 // dinv != NULL: Jacobi-preconditioned CG (p = z = D^-1 r, fused into update and p-update)
 // ||b - A x||^2 and ||b||^2 per segment over the rows but the pinned one, A x accumulated in
-// FP64 (B = 1: K^ms, x and b [n]; B = 9: K^mech, [n][3]): out[2 seg], out[2 seg + 1]
+// FP64 (B = 1: K^ms, x and b [n]; B = 6 or 9: K^mech, [n][3]): out[2 seg], out[2 seg + 1]
 template <typename T>
 cudaError_t launch_true_res(const Launch& L, const DSell& A, const DSeg& G, const T* val, int B,
                             const T* b, const T* x, const T* xlo, Red red, double* out);
