@@ -271,9 +271,10 @@ class Engine final : public EngineBase {
     ST(mem_.alloc(&proj_, 6 * (int64_t)nseg_));
     ST(mem_.alloc(&tres_, 4 * (int64_t)nseg_));
     CK(cudaMemset(tres_, 0, 4 * nseg_ * sizeof(double)));
-    ST(mem_.alloc(&bad_, (int64_t)nseg_));
-    CK(cudaMemset(bad_, 0, nseg_ * sizeof(int)));
-    CK(cudaMallocHost(&host_bad_, nseg_ * sizeof(int)));
+    // (the entry after the last is the fused loops' error flag)
+    ST(mem_.alloc(&bad_, (int64_t)nseg_ + 1));
+    CK(cudaMemset(bad_, 0, (nseg_ + 1) * sizeof(int)));
+    CK(cudaMallocHost(&host_bad_, (nseg_ + 1) * sizeof(int)));
     ST(mem_.alloc(&pinsave_, 3 * (int64_t)nseg_));
     ST(mem_.alloc(&wmean_, n));
     {
@@ -317,6 +318,7 @@ class Engine final : public EngineBase {
     if (!(opt_.flags & GSPM_FLAG_NO_AUTOTUNE)) ST(autotune());
     graph_on_ = (opt_.flags & GSPM_FLAG_GRAPH) != 0;
     if (!hb_.coarse.empty()) ST(init_coarse());
+    ST(init_loop());
     pinned_ = (opt_.flags & GSPM_FLAG_PINNED_CG) ? 1 : 0;
     resolve_ = (opt_.flags & GSPM_FLAG_RESOLVE_AT_MSTAR) != 0;
     return GSPM_OK;
@@ -449,8 +451,9 @@ class Engine final : public EngineBase {
     CK(cudaMemcpyAsync(hz(), host_scal_, 3 * nseg_ * sizeof(double), cudaMemcpyHostToDevice,
                        L_.stream));
     CK(cudaMemsetAsync(bad_, 0, nseg_ * sizeof(int), L_.stream));
-    if (graph_on_ && prof_mask_ == 0) {
-      const int rc = step_graph(n_steps, D, printed, st);
+    const bool graph = graph_on_ && prof_mask_ == 0;
+    if (graph || loop_on_) {
+      const int rc = step_device(n_steps, D, printed, st, graph);
       if (rc != GSPM_OK && rc != GSPM_ENOCONV) return rc;
       ST(check_finite());
       return rc;
@@ -519,10 +522,23 @@ class Engine final : public EngineBase {
     return GSPM_OK;
   }
 
+  // a wait of a fused CG loop gave up: the exchange numbers of its blocks no longer agree, so the
+  // context goes on with the separate kernels
+  int check_loop(int err) {
+    if (!err) return GSPM_OK;
+    loop_on_ = false;
+    ++cfg_gen_;
+    CK(cudaMemsetAsync(bad_ + nseg_, 0, sizeof(int), L_.stream));
+    set_error("a CG loop did not complete within its wait limit");
+    return GSPM_ETIMEOUT;
+  }
+
   int check_finite() {
     ST(check_net());
-    CK(cudaMemcpyAsync(host_bad_, bad_, nseg_ * sizeof(int), cudaMemcpyDeviceToHost, L_.stream));
+    CK(cudaMemcpyAsync(host_bad_, bad_, (nseg_ + 1) * sizeof(int), cudaMemcpyDeviceToHost,
+                       L_.stream));
     CK(cudaStreamSynchronize(L_.stream));
+    ST(check_loop(host_bad_[nseg_]));
     for (int sg = 0; sg < nseg_; ++sg)
       if (host_bad_[sg] > 0) {
         set_error("step: m** not finite or zero at %d magnetic nodes of mesh %d", host_bad_[sg],
@@ -645,16 +661,24 @@ class Engine final : public EngineBase {
         t[2 * nseg_ + 2 * sg + 1] > 0 ? std::sqrt(t[2 * nseg_ + 2 * sg] / t[2 * nseg_ + 2 * sg + 1]) : 0.0;
   }
 
-  int graph_alloc() {
-    if (loop_cnt_) return GSPM_OK;
-    ST(mem_.alloc(&loop_cnt_, kSolveSlots));
+  // device statistics of the graph replays and the fused loops
+  int stats_alloc() {
+    if (gstats_) return GSPM_OK;
     ST(mem_.alloc(&loop_total_, 1));
     ST(mem_.alloc(&gstats_, 4 * (int64_t)nseg_));
-    CK(cudaMemset(loop_cnt_, 0, kSolveSlots * sizeof(int)));
     CK(cudaMemset(loop_total_, 0, sizeof(unsigned long long)));
+    CK(cudaMemset(gstats_, 0, 4 * (size_t)nseg_ * sizeof(long long)));
     const size_t hb = 4 * (size_t)nseg_ * sizeof(long long) + sizeof(unsigned long long) +
                       (size_t)kSolveSlots * nseg_ * sizeof(CGState);
     CK(cudaMallocHost(&host_graph_, hb));
+    return GSPM_OK;
+  }
+
+  int graph_alloc() {
+    if (loop_cnt_) return GSPM_OK;
+    ST(stats_alloc());
+    ST(mem_.alloc(&loop_cnt_, kSolveSlots));
+    CK(cudaMemset(loop_cnt_, 0, kSolveSlots * sizeof(int)));
     CK(cudaStreamCreateWithFlags(&cap_stream_, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&body_stream_, cudaStreamNonBlocking));
     return GSPM_OK;
@@ -755,12 +779,19 @@ class Engine final : public EngineBase {
     return s;
   }
 
-  int step_graph(int n_steps, const DevParams& D, int printed, gspm_step_stats* st) {
-    if (!gexec_ || gexec_x0_ != x0_mode_ || gexec_tres_ != tres_on_ || gexec_gen_ != cfg_gen_)
+  // n_steps without a host round trip: graph replays, or direct launches of the fused CG loops;
+  // the statistics come from the device's accumulators and the last step's CG status blocks
+  int step_device(int n_steps, const DevParams& D, int printed, gspm_step_stats* st, bool graph) {
+    if (graph && (!gexec_ || gexec_x0_ != x0_mode_ || gexec_tres_ != tres_on_ ||
+                  gexec_gen_ != cfg_gen_))
       ST(build_graph(D, printed));
     CK(cudaMemsetAsync(gstats_, 0, 4 * (size_t)nseg_ * sizeof(long long), L_.stream));
-    for (int s = 0; s < n_steps; ++s) CK(cudaGraphLaunch(gexec_, L_.stream));
-    *L_.counter += graph_static_ * n_steps;
+    StepInfo si;
+    for (int s = 0; s < n_steps; ++s) {
+      if (graph) CK(cudaGraphLaunch(gexec_, L_.stream));
+      else ST(step_once(D, printed, &si));
+    }
+    if (graph) *L_.counter += graph_static_ * n_steps;
     long long* hst = reinterpret_cast<long long*>(host_graph_);
     unsigned long long* hloops = reinterpret_cast<unsigned long long*>(hst + 4 * nseg_);
     CGState* hcg = reinterpret_cast<CGState*>(hloops + 1);
@@ -856,6 +887,7 @@ class Engine final : public EngineBase {
     ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, rtol > 0 ? rtol : opt_.rtol_mech, &info));
     TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     if (u) ST(export_field(u_, 1, 3, 3, u, where, ulo_));
+    if (loop_on_) ST(read_mech_info(&info));
     CK(cudaStreamSynchronize(L_.stream));
     int it = 0, nc = 0;
     double rel = 0.0;
@@ -1166,6 +1198,15 @@ class Engine final : public EngineBase {
   // on these operators (5e-5 of ||b|| at 3M nodes)
   static constexpr double kRtolInner = 1e-4;
 
+  // shared memory of a fused loop (227 KB per block less its static part)
+  static constexpr size_t kLoopSmem = 232448 - 4096;
+  // Rows up to which the fused loops run: one mesh, and a batch (whose meshes share the blocks less
+  // evenly and do not converge together).  Mixed precision, ms per step, fused against separate
+  // kernels: 198,400 nodes 12.4 / 22.3, 300,000 15.0 / 23.2, 396,000 20.1 / 26.0, 524,288 25.6 / 29.8;
+  // batches of 252,432 nodes 14.6 / 23.1, 347,296 (FP64) 57.4 / 84.1, 513,808 29.4 / 27.3, 1,138,576
+  // 67.2 / 43.6.
+  static constexpr int64_t kLoopRows = 600000, kLoopBatchRows = 400000;
+
   template <typename X>
   int upload(T** dst, const std::vector<X>& src) {
     ST(mem_.alloc(dst, (int64_t)src.size()));
@@ -1292,7 +1333,7 @@ class Engine final : public EngineBase {
       CK(cudaMemsetAsync(dx_, 0, len * sizeof(T), L_.stream));
       ST(solve_general(slot2, val, B, b, x, dx_, rtol, &i2));
       TK(GSPM_KCLASS_CG_INIT, launch_refine_add<T>(L_, len, x, xlo, dx_));
-      if (!capturing_) {
+      if (!capturing_ && !loop_on_) {
         info->assign(nseg_, SolveInfo());
         for (int sg = 0; sg < nseg_; ++sg) {
           (*info)[sg].iters = i1[sg].iters + i2[sg].iters;
@@ -1345,6 +1386,16 @@ class Engine final : public EngineBase {
       return GSPM_OK;
     };
     TK(GSPM_KCLASS_CG_INIT, launch_cg_init<T>(L_, A_, SG_, val, B, b, x0, r_, p_, st, na, rtol, opt_.max_iter, red_, pinned_ ? nullptr : bmean, pinned_, pc ? 1 : 0));
+    if (loop_on_) {
+      if (!pinned_ && !pc) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
+      CgLoop<T> a = loop_args(slot, val, len, x, dinv, B == 1 ? 0 : 1);
+      a.pinned = pinned_;
+      a.shift = !pinned_;
+      const int npc = pc ? 1 : 0;
+      a.place = loop_place(epr, 1, npc);
+      TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_loop<T>(L_, a, B, 1, npc));
+      return GSPM_OK;
+    }
     if (pc) ST(precondition(p_, 1));
     // singular system: p0 projected off the constants
     if (!pinned_) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
@@ -1380,6 +1431,13 @@ class Engine final : public EngineBase {
     CK(cudaMemsetAsync(na, 0, sizeof(int), L_.stream));
     const T* dinv = aval == Aeps_ ? dgs_eps_ : dgs_aeps_;  // NULL: plain CG
     TK(GSPM_KCLASS_CG_INIT, launch_cg_init_gs<T>(L_, A_, SG_, aval, M_, nr, ld_, x, r_, p_, st, na, opt_.rtol_gs, opt_.max_iter, red_, dinv));
+    if (loop_on_) {
+      CgLoop<T> a = loop_args(slot, aval, ld_, x, dinv, 2);
+      const int npc = dinv ? 2 : 0;
+      a.place = loop_place(1, nr, npc);
+      TK(GSPM_KCLASS_SPMV_GS, launch_cg_loop<T>(L_, a, 1, nr, npc));
+      return GSPM_OK;
+    }
     auto iter = [&]() -> int {
       TK(GSPM_KCLASS_SPMV_GS, launch_cg_spmv<T>(L_, A_, SG_, aval, 1, nr, ld_, p_, q_, st, red_, var_gs_, 0, 0));
       TK(GSPM_KCLASS_CG_VEC, launch_cg_update<T>(L_, SG_, 1, nr, ld_, x, r_, p_, q_, st, na, red_, dinv));
@@ -1398,6 +1456,217 @@ class Engine final : public EngineBase {
         info[k][sg].noconv = k == 0 ? tot[sg].noconv : 0;
       }
     }
+    return GSPM_OK;
+  }
+
+  // ---------------------------------------------------------------- fused CG loops (cgloop.cu)
+  // iterations and residual of the last K^mech solve, from the device (synchronises)
+  int read_mech_info(std::vector<SolveInfo>* info) {
+    CGState* h = static_cast<CGState*>(host_graph_);
+    CK(cudaMemcpyAsync(h, cg_, (size_t)kSolveSlots * nseg_ * sizeof(CGState),
+                       cudaMemcpyDeviceToHost, L_.stream));
+    CK(cudaMemcpyAsync(host_bad_ + nseg_, bad_ + nseg_, sizeof(int), cudaMemcpyDeviceToHost,
+                       L_.stream));
+    CK(cudaStreamSynchronize(L_.stream));
+    ST(check_loop(host_bad_[nseg_]));
+    info->assign(nseg_, SolveInfo());
+    for (int sg = 0; sg < nseg_; ++sg) {
+      (*info)[sg] = info_of(h[kSlotMech * nseg_ + sg], -1);
+      if (!ulo_) continue;
+      const SolveInfo i2 = info_of(h[kSlotMech2 * nseg_ + sg], -1);
+      (*info)[sg].iters += i2.iters;
+      (*info)[sg].relres = i2.relres;
+      (*info)[sg].noconv += i2.noconv;
+    }
+    return GSPM_OK;
+  }
+
+  CgLoop<T> loop_args(int slot, const T* val, int64_t ld, T* x, const T* dinv, int kind) const {
+    CgLoop<T> a{};
+    a.A = A_;
+    a.G = SG_;
+    a.C = CC_;
+    a.part = LP_;
+    a.val = val;
+    a.ld = ld;
+    a.x = x;
+    a.r = r_;
+    a.p = p_;
+    a.q = q_;
+    a.dinv = dinv;
+    a.st = cg_ + (int64_t)slot * nseg_;
+    a.acc = gstats_;
+    a.kind = kind;
+    return a;
+  }
+
+  // how many of the vectors r, q, p, x, D^-1 fit the shared memory beside the rest
+  int loop_place(int nc, int nr, int pc) const {
+    int k = 5;
+    while (k > 0 && loop_smem<T>(nc, nr, pc, k, LP_).total > kLoopSmem) --k;
+    return k;
+  }
+
+  // Rows to blocks for the fused loops, or loop_on_ = false where they do not apply: aggregates
+  // that are not runs of rows, more meshes than blocks, operators without symmetric blocks, or
+  // a size at which the separate kernels are as fast (see kLoopRows).
+  int init_loop() {
+    const int S = nseg_;
+    const int max_blocks = std::min(L_.sms, kLoopMaxBlocks);
+    int coop = 0, dev = 0;
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+    if (!coop || kb_ != 6 || S > max_blocks || n_ > (S == 1 ? kLoopRows : kLoopBatchRows))
+      return GSPM_OK;
+    if (pc_ && !CC_.contig) return GSPM_OK;
+    // blocks per mesh: one each, the rest to whichever mesh has the most slices per block
+    std::vector<int64_t> nb(S, 1);
+    for (int left = max_blocks - S; left > 0; --left) {
+      int best = -1;
+      for (int sg = 0; sg < S; ++sg)
+        if (nb[sg] < hb_.seg_nsl[sg] &&
+            (best < 0 || hb_.seg_nsl[sg] * nb[best] > hb_.seg_nsl[best] * nb[sg]))
+          best = sg;
+      if (best < 0) break;
+      ++nb[best];
+    }
+    std::vector<int32_t> seg, sl0, sl1, segb(S + 1, 0), pinb(S, 0), pc0, ap;
+    std::vector<int64_t> prow;
+    int64_t max_sl = 0, min_sl = INT64_MAX;
+    int max_pieces = 0, max_aggp = 0, max_ldc[2] = {0, 0};
+    std::vector<int32_t> agg0(S + 1, 0);
+    if (pc_) {
+      for (int sg = 0; sg < S; ++sg) agg0[sg + 1] = agg0[sg] + (int32_t)hb_.coarse[sg].n_agg;
+      ap.assign(agg0[S] + 1, 0);
+    }
+    for (int sg = 0; sg < S; ++sg) {
+      segb[sg] = (int32_t)seg.size();
+      const int64_t nsl = hb_.seg_nsl[sg], rend = hb_.seg_row0[sg] + hb_.seg_nrow[sg];
+      const size_t p_seg = prow.size();
+      int32_t last = -1;
+      for (int64_t i = 0; i < nb[sg]; ++i) {
+        const int64_t a = hb_.seg_sl0[sg] + i * nsl / nb[sg];
+        const int64_t b = hb_.seg_sl0[sg] + (i + 1) * nsl / nb[sg];
+        max_sl = std::max(max_sl, b - a);
+        min_sl = std::min(min_sl, b - a);
+        if (hb_.seg_pin[sg] >= a * 32 && hb_.seg_pin[sg] < b * 32) pinb[sg] = (int32_t)seg.size();
+        seg.push_back(sg);
+        sl0.push_back((int32_t)a);
+        sl1.push_back((int32_t)b);
+        pc0.push_back((int32_t)prow.size());
+        if (!pc_) continue;
+        const std::vector<int32_t>& agg = hb_.coarse[sg].agg;
+        for (int64_t row = a * 32; row < std::min(b * 32, rend); ++row) {
+          const int32_t I = agg[row - hb_.seg_row0[sg]];
+          if (I != last && I != last + 1) return GSPM_OK;  // not numbered in row order
+          if (I == last && row > a * 32) continue;
+          prow.push_back(row);
+          ++ap[agg0[sg] + I + 1];
+          last = I;
+        }
+        max_pieces = std::max(max_pieces, (int)prow.size() - pc0.back());
+      }
+      max_aggp = std::max(max_aggp, (int)(prow.size() - p_seg));
+    }
+    segb[S] = (int32_t)seg.size();
+    pc0.push_back((int32_t)prow.size());
+    for (size_t I = 1; I < ap.size(); ++I) ap[I] += ap[I - 1];
+    LoopPart P{};
+    P.nblocks = (int)seg.size();
+    P.max_rows = (int)(32 * max_sl);
+    P.min_slices = (int)min_sl;
+    P.max_pieces = max_pieces;
+    P.max_aggp = max_aggp;
+    using S16 = typename CoarseStore<T>::type;
+    constexpr int64_t W = 16 / sizeof(S16);  // rows padded to whole 16-byte packs
+    if (pc_)
+      for (int e = 0; e < 2; ++e)
+        for (int sg = 0; sg < S; ++sg) {
+          const int64_t nc = (e == 0 ? 3 : 1) * hb_.coarse[sg].n_agg;
+          max_ldc[e] = std::max(max_ldc[e], (int)((nc + W - 1) / W * W));
+        }
+    P.max_ldc[0] = max_ldc[0];
+    P.max_ldc[1] = max_ldc[1];
+    for (int nc = 1; nc <= 3; nc += 2)
+      if (loop_smem<T>(nc, 1, pc_ ? 1 : 0, 0, P).total > kLoopSmem) return GSPM_OK;
+    if (loop_smem<T>(1, 3, 2, 0, P).total > kLoopSmem) return GSPM_OK;
+    auto up = [&](auto** dst, const auto& v) -> int {
+      ST(mem_.alloc(dst, (int64_t)v.size()));
+      CK(cudaMemcpy(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice));
+      return GSPM_OK;
+    };
+    int32_t *d_seg, *d_sl0, *d_sl1, *d_segb, *d_pinb;
+    ST(up(&d_seg, seg));
+    ST(up(&d_sl0, sl0));
+    ST(up(&d_sl1, sl1));
+    ST(up(&d_segb, segb));
+    ST(up(&d_pinb, pinb));
+    P.seg = d_seg;
+    P.sl0 = d_sl0;
+    P.sl1 = d_sl1;
+    P.seg_b0 = d_segb;
+    P.pin_blk = d_pinb;
+    if (pc_) {
+      int32_t *d_pc0, *d_ap;
+      int64_t* d_prow;
+      ST(up(&d_pc0, pc0));
+      ST(up(&d_ap, ap));
+      ST(up(&d_prow, prow));
+      P.pc0 = d_pc0;
+      P.ap = d_ap;
+      P.pc_row = d_prow;
+      for (int e = 0; e < 2; ++e) {
+        std::vector<int64_t> off(S);
+        std::vector<int32_t> ldv(S);
+        int64_t total = 0;
+        for (int sg = 0; sg < S; ++sg) {
+          const int64_t nc = (e == 0 ? 3 : 1) * hb_.coarse[sg].n_agg, l = (nc + W - 1) / W * W;
+          off[sg] = total;
+          ldv[sg] = (int32_t)l;
+          total += nc * l;
+        }
+        std::vector<S16> data(total, S16(0));
+        for (int sg = 0; sg < S; ++sg) {
+          const HostCoarse& hc = hb_.coarse[sg];
+          const std::vector<double>& inv = e == 0 ? hc.store_mech : hc.store_ms;
+          const int64_t nc = (e == 0 ? 3 : 1) * hc.n_agg;
+          for (int64_t i = 0; i < nc; ++i)
+            for (int64_t j = 0; j < nc; ++j)
+              data[off[sg] + i * ldv[sg] + j] = to_store<S16>(inv[i * nc + j]);
+        }
+        S16* d_inv;
+        int64_t* d_off;
+        int32_t* d_ld;
+        ST(up(&d_inv, data));
+        ST(up(&d_off, off));
+        ST(up(&d_ld, ldv));
+        P.inv[e] = d_inv;
+        P.inv_off[e] = d_off;
+        P.inv_ld[e] = d_ld;
+      }
+    }
+    const int64_t ex = kLoopExchanges * kLoopExStride, ln = kLoopLineKinds * kLoopLines;
+    const int64_t rc = 3 * (int64_t)prow.size(), ec = 3 * (int64_t)agg0[S];
+    char* pp = nullptr;
+    ST(mem_.alloc(&P.epoch, 2 * S));
+    ST(mem_.alloc(&P.count, S));
+    ST(mem_.alloc(&P.ex, ex));
+    ST(mem_.alloc(&P.line, ln));
+    ST(mem_.alloc(&P.rcx, rc));
+    ST(mem_.alloc(&P.ecx, ec));
+    ST(mem_.alloc(&pp, 3 * ld_ * 2 * (int64_t)sizeof(T)));
+    P.pp = pp;
+    CK(cudaMemset(P.epoch, 0, 2 * S * sizeof(uint32_t)));
+    CK(cudaMemset(P.count, 0, S * sizeof(uint32_t)));
+    CK(cudaMemset(P.ex, 0, ex * sizeof(ulonglong2)));
+    CK(cudaMemset(P.line, 0, ln * sizeof(ulonglong2)));
+    CK(cudaMemset(P.rcx, 0, std::max<int64_t>(1, rc) * sizeof(ulonglong2)));
+    CK(cudaMemset(P.ecx, 0, std::max<int64_t>(1, ec) * sizeof(ulonglong2)));
+    CK(cudaMemset(P.pp, 0, 3 * ld_ * 2 * sizeof(T)));
+    P.err = bad_ + nseg_;
+    LP_ = P;
+    ST(stats_alloc());
+    loop_on_ = true;
     return GSPM_OK;
   }
 
@@ -1845,6 +2114,9 @@ class Engine final : public EngineBase {
   T *dinv3_ = nullptr, *dinv1_ = nullptr;
   T *dgs_eps_ = nullptr, *dgs_aeps_ = nullptr;  // Jacobi of the GSPM solves (NULL: plain)
   T *rc_ = nullptr, *ec_ = nullptr;
+  // fused CG loops
+  LoopPart LP_{};
+  bool loop_on_ = false;
   // CUDA-graph replay state
   bool graph_on_ = false, capturing_ = false;
   cudaStream_t cap_stream_ = nullptr, body_stream_ = nullptr;

@@ -297,4 +297,95 @@ template <typename T>
 cudaError_t launch_scaled_diff(const Launch& L, int64_t len, const T* a, const T* b, const T* c,
                                double scale, float* t);
 
+// ---- a whole CG loop in one cooperative kernel (cgloop.cu) -----------------------------------
+constexpr int kLoopThreads = 512;
+constexpr int kLoopMaxBlocks = 160;                  // one block per SM (152)
+constexpr int kLoopExStride = 8 * kLoopMaxBlocks;    // packets of one exchange: [value][block]
+constexpr int kLoopExchanges = 3;
+constexpr int kLoopLines = 8 * kLoopMaxBlocks;       // packets of one kind of line: [block][value]
+constexpr int kLoopLineKinds = 3;
+// coarse unknowns squared per server block: its share of the dense product then takes some 500
+// cycles (FP64: two multiply-adds per clock and SM)
+template <typename T>
+constexpr int64_t kLoopServe = sizeof(T) == 4 ? 8192 : 1024;
+
+// Rows to blocks: block b owns the slices [sl0[b], sl1[b]) of segment seg[b]; segment s has the
+// blocks [seg_b0[s], seg_b0[s + 1]).  A piece is the part of one aggregate in one block (rows are
+// numbered aggregate by aggregate): block b's pieces are [pc0[b], pc0[b + 1]), piece k starts at row
+// pc_row[k], aggregate I's pieces are [ap[I], ap[I + 1]).  inv: the dense coarse inverses, full and
+// row-major, rows padded to inv_ld values, segment s at inv_off[s] ([0]: K^mech, [1]: K^ms).
+struct LoopPart {
+  int nblocks, max_rows;      // most rows of a block (whole slices)
+  int min_slices;             // fewest slices of a block
+  int max_pieces, max_aggp;   // most pieces of a block, of a segment
+  int max_ldc[2];             // longest padded row of the coarse inverses
+  const int32_t *seg, *sl0, *sl1;
+  const int32_t* seg_b0;
+  const int32_t* pin_blk;     // [nseg] block that owns the pinned row
+  const int32_t *pc0, *ap;
+  const int64_t* pc_row;
+  const void* inv[2];
+  const int64_t* inv_off[2];
+  const int32_t* inv_ld[2];
+  uint32_t* epoch;            // [nseg][2] numbers of the last exchange and the last barrier
+  uint32_t* count;            // [nseg] arrivals at barriers
+  ulonglong2* ex;             // [kLoopExchanges * kLoopExStride] sums for the leaders
+  ulonglong2* line;           // [kLoopLineKinds * kLoopLines] scalars from the leaders
+  ulonglong2* rcx;            // [3 * pieces] restricted residual
+  ulonglong2* ecx;            // [3 * aggregates] coarse correction
+  void* pp;                   // [3 * ld] p as packets (8 bytes per value in FP32, 16 in FP64)
+  int* err;                   // set when a wait gave up
+};
+
+template <typename T>
+struct CgLoop {
+  DSell A;
+  DSeg G;
+  DCoarse C;
+  LoopPart part;
+  const T* val;
+  int64_t ld;                 // stride between right-hand sides (scalar rows)
+  T *x, *r, *p, *q;           // q: scratch
+  const T* dinv;
+  CGState* st;
+  long long* acc;             // statistics (see launch_solve_stats)
+  int kind, pinned, shift;    // shift: move x to zero at the pinned row
+  int place;                  // of r, q, p, x, D^-1 the first `place` live in shared memory
+};
+
+// Shared memory of a loop kernel, byte offsets
+struct LoopSmem {
+  int comb, psum, pieces, rc, ec, prow, vec[5];
+  size_t total;
+};
+template <typename T>
+__host__ __device__ inline LoopSmem loop_smem(int nc, int nr, int pc, int place,
+                                              const LoopPart& P) {
+  LoopSmem m;
+  size_t o = 0;
+  const size_t w = sizeof(T);
+  const int nv = nc == 3 ? 3 : nr;
+  const int ldc = P.max_ldc[nc == 3 ? 0 : 1];
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o += (bytes + 15) / 16 * 16;
+    return (int)at;
+  };
+  // (only blocks whose slices several warps share combine partial rows)
+  m.comb = take(2 * P.min_slices <= kLoopThreads / 32 ? (size_t)kLoopThreads * nv * w : 0);
+  m.psum = take(pc == 1 ? (size_t)P.max_pieces * (kLoopThreads / 32) * nc * w : 0);
+  m.pieces = take(pc == 1 ? (size_t)P.max_aggp * nc * w : 0);
+  m.rc = take(pc == 1 ? (size_t)ldc * w : 0);
+  m.ec = take(pc == 1 ? (size_t)P.max_pieces * nc * w : 0);
+  m.prow = take(pc == 1 ? (size_t)(P.max_pieces + 1) * 4 : 0);
+  for (int k = 0; k < 5; ++k)
+    m.vec[k] = take(k < place ? (size_t)P.max_rows * (k == 4 ? nc : nv) * w : 0);
+  m.total = o;
+  return m;
+}
+// B = 1 (kind 0: K^ms; kind 2: GSPM, nr right-hand sides) or 6 (K^mech); pc: 0 plain, 1 two-level,
+// 2 Jacobi
+template <typename T>
+cudaError_t launch_cg_loop(const Launch& L, const CgLoop<T>& a, int B, int nr, int pc);
+
 }  // namespace gspm
