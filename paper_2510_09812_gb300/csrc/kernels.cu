@@ -18,6 +18,7 @@
 #include <unordered_map>
 
 #include "device.cuh"
+#include "flatsum.cuh"
 #include "kernels.cuh"
 
 namespace gspm {
@@ -25,33 +26,43 @@ namespace gspm {
 namespace {
 
 // ------------------------------------------------------------------------------------------
-// volume average per segment: out[seg*nc + c] = sum_i w_i f(i, c) (+ add[c]); Sec. 2.4 with
+// volume average per segment: out[seg*NC + c] = sum_i w_i f(i, c) (+ add[c]); Sec. 2.4 with
 // nodal weights M_L,i / V(segment)
 // ------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_wsum(DSeg G, ItemList IL, int nc, const T* __restrict__ f,
+template <typename T, int NC>
+__global__ void __launch_bounds__(kBlock) k_wsum(DSeg G, ItemList IL, const T* __restrict__ f,
                                                  int64_t cs, int64_t ns,
-                                                 const int64_t* __restrict__ perm,
                                                  const double* __restrict__ w, double* out,
                                                  const double* add, Red red) {
   for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
     const int seg = IL.seg[item];
-    double v[9];
+    double v[NC];
 #pragma unroll
-    for (int c = 0; c < 9; ++c) v[c] = 0.0;
+    for (int c = 0; c < NC; ++c) v[c] = 0.0;
     const int64_t r0 = (int64_t)IL.sl0[item] * 32, r1 = (int64_t)IL.sl1[item] * 32;
     for (int64_t i = r0 + threadIdx.x; i < r1; i += blockDim.x) {
       if (!row_valid(G, seg, i)) continue;
       const double wi = w[i];
-      const int64_t src = perm ? perm[i] : i;
 #pragma unroll
-      for (int c = 0; c < 9; ++c)
-        if (c < nc) v[c] += wi * (double)f[src * ns + c * cs];
+      for (int c = 0; c < NC; ++c) v[c] += wi * (double)f[i * ns + c * cs];
     }
-    __shared__ double res[9];
-    if (seg_reduce<9>(v, item, seg, G, IL, red, res) && threadIdx.x == 0)
-      for (int c = 0; c < nc; ++c) out[seg * nc + c] = res[c] + (add ? add[c] : 0.0);
+    __shared__ double res[NC];
+    if (seg_reduce<NC>(v, item, seg, G, IL, red, res) && threadIdx.x == 0)
+      for (int c = 0; c < NC; ++c) out[seg * NC + c] = res[c] + (add ? add[c] : 0.0);
   }
+}
+
+// the same for a field in ABI order ([nodes][nc] float64), one grid row per segment
+__global__ void __launch_bounds__(kSumThreads) k_volume_avg(const int64_t* __restrict__ node0,
+                                                            const int64_t* __restrict__ count,
+                                                            int nc, const double* __restrict__ f,
+                                                            const double* __restrict__ w,
+                                                            double* out, double* partials,
+                                                            unsigned* counter) {
+  const int seg = blockIdx.y;
+  const int64_t i0 = node0[seg];
+  flat_sum(count[seg], nc, f + i0 * nc, w + i0, out + seg * nc,
+           partials + (int64_t)seg * kSumGrid * kSumComp, counter + seg);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1679,14 +1690,33 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), int grid, cudaStream_t stream
 #define GSPM_GRID(L, threads, kern) grid_for((L), (threads), reinterpret_cast<const void*>(kern))
 #define GSPM_IGRID(L, G, kern) item_grid((L), (G), reinterpret_cast<const void*>(kern))
 
+template <typename T, int NC>
+static cudaError_t wsum_nc(const Launch& L, const DSeg& G, const T* f, int64_t cs, int64_t ns,
+                           const double* w, double* out, const double* add, Red red) {
+  auto k = k_wsum<T, NC>;
+  const ItemGrid ig = GSPM_IGRID(L, G, k);
+  k<<<ig.grid, kBlock, 0, L.stream>>>(G, ig.list, f, cs, ns, w, out, add, red);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_wsum(const Launch& L, const DSeg& G, int nc, const T* f, int64_t cs,
-                        int64_t ns, const int64_t* perm, const double* w, double* out,
-                        const double* add, Red red) {
+                        int64_t ns, const double* w, double* out, const double* add, Red red) {
   (*L.counter) += 1;
-  auto k = k_wsum<T>;
-  const ItemGrid ig = GSPM_IGRID(L, G, k);
-  k<<<ig.grid, kBlock, 0, L.stream>>>(G, ig.list, nc, f, cs, ns, perm, w, out, add, red);
+  switch (nc) {
+    case 1: return wsum_nc<T, 1>(L, G, f, cs, ns, w, out, add, red);
+    case 3: return wsum_nc<T, 3>(L, G, f, cs, ns, w, out, add, red);
+    case 6: return wsum_nc<T, 6>(L, G, f, cs, ns, w, out, add, red);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_volume_avg(const Launch& L, int nseg, int64_t max_nodes, const int64_t* node0,
+                              const int64_t* count, int nc, const double* f, const double* w,
+                              double* out, double* partials, unsigned* counter) {
+  (*L.counter) += 1;
+  k_volume_avg<<<dim3((unsigned)sum_blocks(max_nodes, nc), (unsigned)nseg), kSumThreads, 0,
+                 L.stream>>>(node0, count, nc, f, w, out, partials, counter);
   return cudaGetLastError();
 }
 
@@ -2176,8 +2206,7 @@ cudaError_t launch_scaled_diff(const Launch& L, int64_t len, const T* a, const T
 
 #define GSPM_INSTANTIATE(T)                                                                       \
   template cudaError_t launch_wsum<T>(const Launch&, const DSeg&, int, const T*, int64_t,        \
-                                      int64_t, const int64_t*, const double*, double*,            \
-                                      const double*, Red);                                        \
+                                      int64_t, const double*, double*, const double*, Red);       \
   template cudaError_t launch_spmv<T>(const Launch&, const DSell&, const T*, int, const T*, T*,   \
                                       int, int);                                                  \
   template cudaError_t launch_cg_init<T>(const Launch&, const DSell&, const DSeg&, const T*, int, \
