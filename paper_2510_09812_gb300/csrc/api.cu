@@ -166,6 +166,7 @@ class Engine final : public EngineBase {
     if (host_active_) cudaFreeHost(host_active_);
     if (host_scal_) cudaFreeHost(host_scal_);
     if (host_avg_) cudaFreeHost(host_avg_);
+    if (host_grad_) cudaFreeHost(host_grad_);
     for (cudaEvent_t e : prof_ev_) cudaEventDestroy(e);
   }
 
@@ -518,11 +519,12 @@ class Engine final : public EngineBase {
     int e = 0;
     CK(cudaMemcpyAsync(&e, mpnn_err_, sizeof(int), cudaMemcpyDeviceToHost, L_.stream));
     CK(cudaStreamSynchronize(L_.stream));
-    if (e) {
-      set_error("learned initial guess: a tensor-core layer did not complete within its wait limit");
-      return GSPM_ETIMEOUT;
-    }
-    return GSPM_OK;
+    return net_error(e);
+  }
+  int net_error(int e) const {
+    if (!e) return GSPM_OK;
+    set_error("learned initial guess: a tensor-core layer did not complete within its wait limit");
+    return GSPM_ETIMEOUT;
   }
 
   // a wait of a fused CG loop gave up: the exchange numbers of its blocks no longer agree, so the
@@ -1162,12 +1164,15 @@ class Engine final : public EngineBase {
       return GSPM_EINVAL;
     }
     ST(net_step(pair, /*update=*/false, 0.0));
-    float l = 0.f;
-    CK(cudaMemcpyAsync(&l, loss_, sizeof(float), cudaMemcpyDeviceToHost, L_.stream));
-    if (grad) CK(cudaMemcpyAsync(grad, grad_, kParams * sizeof(float), cudaMemcpyDeviceToHost, L_.stream));
+    // gradient, loss and the layers' error flag lie together: one copy, to pinned memory
+    CK(cudaMemcpyAsync(host_grad_, grad_, (kParams + 2) * sizeof(float), cudaMemcpyDeviceToHost,
+                       L_.stream));
     CK(cudaStreamSynchronize(L_.stream));
-    ST(check_net());
-    if (loss) *loss = (double)l / (3.0 * (double)n_);
+    int err = 0;
+    memcpy(&err, host_grad_ + kParams + 1, sizeof(int));
+    ST(net_error(err));
+    if (grad) memcpy(grad, host_grad_, kParams * sizeof(float));
+    if (loss) *loss = (double)host_grad_[kParams] / (3.0 * (double)n_);
     return GSPM_OK;
   }
 
@@ -1945,10 +1950,13 @@ class Engine final : public EngineBase {
     }
     CK(mpnn_setup_smem());
     ST(mem_.alloc(&params_, kParams));
-    ST(mem_.alloc(&grad_, kParams));
+    ST(mem_.alloc(&grad_, kParams + 2));  // then the loss and the error flag
+    CK(cudaMemset(grad_, 0, (kParams + 2) * sizeof(float)));
+    CK(cudaMallocHost(&host_grad_, (kParams + 2) * sizeof(float)));
+    loss_ = grad_ + kParams;
+    mpnn_err_ = reinterpret_cast<int*>(grad_ + kParams + 1);
     ST(mem_.alloc(&adam_m_, kParams));
     ST(mem_.alloc(&adam_v_, kParams));
-    ST(mem_.alloc(&loss_, 4));
     ST(mem_.alloc(&WinT_, kHid * kFeat));
     for (int l = 0; l < kLayers; ++l) ST(mem_.alloc(&WT_[l], kHid * 2 * kHid));
     ST(mem_.alloc(&F_in_, n_ * kFeat));
@@ -1965,8 +1973,6 @@ class Engine final : public EngineBase {
     net_.bout = params_ + kOffBout;
     net_.A = agg_;
     net_.At = aggT_;
-    ST(mem_.alloc(&mpnn_err_, 1));
-    CK(cudaMemset(mpnn_err_, 0, sizeof(int)));
     net_.err = mpnn_err_;
     return GSPM_OK;
   }
@@ -2058,6 +2064,7 @@ class Engine final : public EngineBase {
   int adam_t_ = 0, ds_cap_ = 0, ds_n_ = 0;
   MpnnDev net_{};
   int* mpnn_err_ = nullptr;
+  float* host_grad_ = nullptr;  // pinned
   T *u2_ = nullptr, *utmp_ = nullptr, *uin_ = nullptr, *uin2_ = nullptr;
 
   // launch f() bracketed by CUDA events when class cls is being profiled

@@ -427,151 +427,281 @@ __global__ void __launch_bounds__(kThreads) k_out_bwd(int64_t n, const float* __
     part[(int64_t)blockIdx.x * (kHid * 3 + 4) + k] = acc[k];
 }
 
+// Rows of a backward tile and the padded row lengths of its shared arrays (multiples of four floats,
+// so that rows of consecutive lanes start four banks apart: 16-byte accesses without conflicts)
+constexpr int kBwdRows = 64;
+constexpr int kPitch = kHid + 4, kPitch2 = 2 * kHid + 4;
+
+// 16 consecutive bf16 values
+__device__ __forceinline__ void load16(const __nv_bfloat16* p, float (&v)[16]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint4 u = *reinterpret_cast<const uint4*>(p + 8 * h);
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[8 * h + 2 * k] = __uint_as_float(w[k] << 16);
+      v[8 * h + 2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+    }
+  }
+}
+__device__ __forceinline__ void store16(float* p, const float (&v)[16]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    *reinterpret_cast<float4*>(p + 4 * k) =
+        make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+}
+// dA = dH (.) [h > 0], 16 columns from c0 of row i (zero past the last row)
+__device__ __forceinline__ void load_da(int64_t n, int64_t i, int c0, const float* __restrict__ dH,
+                                        const __nv_bfloat16* __restrict__ H, float (&v)[16]) {
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = 0.f;
+  if (i >= n) return;
+  float h[16];
+  load16(H + i * kHid + c0, h);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 d = *reinterpret_cast<const float4*>(dH + i * kHid + c0 + 4 * k);
+    v[4 * k] = h[4 * k] > 0.f ? d.x : 0.f;
+    v[4 * k + 1] = h[4 * k + 1] > 0.f ? d.y : 0.f;
+    v[4 * k + 2] = h[4 * k + 2] > 0.f ? d.z : 0.f;
+    v[4 * k + 3] = h[4 * k + 3] > 0.f ? d.w : 0.f;
+  }
+}
+
 // For one layer: dA = dH (.) [h > 0]; block partials of dW (X^T dA, X = [h_prev, z]) and db;
-// dXself = dA W^T[:, :64] -> dHprev, dZ = dA W^T[:, 64:]
-__global__ void __launch_bounds__(kThreads) k_layer_bwd(int64_t n, const float* __restrict__ dH,
-                                                        const __nv_bfloat16* __restrict__ Hcur,
-                                                        const __nv_bfloat16* __restrict__ Hprev,
-                                                        const __nv_bfloat16* __restrict__ Z,
-                                                        const float* __restrict__ W,  // [128][64]
-                                                        float* __restrict__ dHprev,
-                                                        float* __restrict__ dZ,
-                                                        float* __restrict__ part) {
+// dX = dA W^T: columns 0..63 -> dHprev, 64..127 -> dZ.  Both products of a tile of 64 rows are
+// register-tiled FP32 (32 outputs per thread from three 16-byte shared loads per step; a tile's part
+// of dW is summed by itself before it joins the block's running sum).  The FP32 pipe bounds it: 29 us
+// at 65,536 rows, of which the 1,024 tiles fill 304 blocks in four rounds where 3.4 would do; it takes
+// 63 us, against 209 us with two shared loads per multiply-add.
+__global__ void __launch_bounds__(kThreads, 2) k_layer_bwd(int64_t n, const float* __restrict__ dH,
+                                                           const __nv_bfloat16* __restrict__ Hcur,
+                                                           const __nv_bfloat16* __restrict__ Hprev,
+                                                           const __nv_bfloat16* __restrict__ Z,
+                                                           const float* __restrict__ W,  // [128][64]
+                                                           float* __restrict__ dHprev,
+                                                           float* __restrict__ dZ,
+                                                           float* __restrict__ part) {
   // part per block: [128*64 dW][64 db]
   extern __shared__ __align__(16) unsigned char smem[];
-  float* WsT = reinterpret_cast<float*>(smem);          // [64][128]: WsT[c][f] = W[f][c]
-  float* Xr = WsT + 2 * kHid * kHid;                    // [8 warps][128]
-  float* Dr = Xr + 8 * 2 * kHid;                        // [8 warps][64]
-  for (int k = threadIdx.x; k < 2 * kHid * kHid; k += blockDim.x)
-    WsT[(k % kHid) * 2 * kHid + k / kHid] = W[k];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // each thread owns dW entries (f, c) for f in {lane + 32 q}, c in {2 warp .. } ... use a
-  // simple ownership: thread k owns 32 consecutive entries of the flattened [128][64] block
-  float pw[32];
-  for (int q = 0; q < 32; ++q) pw[q] = 0.f;
-  float pb[2] = {0.f, 0.f};
-  const int64_t nwarps = tstride() >> 5;
-  // rows are processed warp-synchronously in rounds so that every warp's row is staged before
-  // the block-wide dW accumulation of that round
-  const int64_t rounds = (n + nwarps - 1) / nwarps;
-  for (int64_t rd = 0; rd < rounds; ++rd) {
-    const int64_t i = rd * nwarps + (tid() >> 5);
-    float* xr = Xr + warp * 2 * kHid;
-    float* dr = Dr + warp * kHid;
-    if (i < n) {
-      for (int c = lane; c < kHid; c += 32) {
-        const float hc = bf(Hcur + i * kHid + c);
-        const float d = hc > 0.f ? dH[i * kHid + c] : 0.f;
-        dr[c] = d;
-        xr[c] = bf(Hprev + i * kHid + c);
-        xr[kHid + c] = bf(Z + i * kHid + c);
+  float* WT = reinterpret_cast<float*>(smem);  // [64][kPitch2]: WT[c][f] = W[f][c]
+  float* X = WT + kHid * kPitch2;              // [rows][kPitch2]
+  float* D = X + kBwdRows * kPitch2;           // [rows][kPitch]   dA
+  float* DT = D + kBwdRows * kPitch;           // [64][kPitch]     its transpose
+  const int t = threadIdx.x;
+  for (int k = t; k < 2 * kHid * kHid; k += kThreads) WT[(k % kHid) * kPitch2 + k / kHid] = W[k];
+  const int lr = t % kBwdRows, lc = 16 * (t / kBwdRows);  // loads: row and first column
+  const int tx = 4 * (t % 16), ty = 4 * (t / 16);
+  float w[2][4][4] = {}, db = 0.f;  // dW[64 h + ty + i][tx + j]
+  for (int64_t base = (int64_t)blockIdx.x * kBwdRows; base < n;
+       base += (int64_t)gridDim.x * kBwdRows) {
+    const int64_t i = base + lr;
+    float v[16];
+    load_da(n, i, lc, dH, Hcur, v);
+    __syncthreads();  // the tile before has been read
+    store16(D + lr * kPitch + lc, v);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) DT[(lc + k) * kPitch + lr] = v[k];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (i < n) {
+        load16((h ? Z : Hprev) + i * kHid + lc, v);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = 0.f;
       }
-    } else {
-      for (int c = lane; c < kHid; c += 32) {
-        dr[c] = 0.f;
-        xr[c] = 0.f;
-        xr[kHid + c] = 0.f;
-      }
-    }
-    __syncwarp();
-    if (i < n) {
-      // dX[f] = sum_c dA[c] W[f][c], f = lane + 32 q
-      for (int q = 0; q < 4; ++q) {
-        const int f = lane + 32 * q;
-        float s = 0.f;
-        for (int c = 0; c < kHid; ++c) s += dr[c] * WsT[c * 2 * kHid + f];
-        if (f < kHid)
-          dHprev[i * kHid + f] = s;
-        else
-          dZ[i * kHid + f - kHid] = s;
-      }
-      pb[0] += dr[lane];
-      pb[1] += dr[lane + 32];
+      store16(X + lr * kPitch2 + h * kHid + lc, v);
     }
     __syncthreads();
-    // dW[f][c] += sum over the round's rows of X[f] dA[c]; thread t owns entries 32t .. 32t+31
-    for (int w8 = 0; w8 < 8; ++w8) {
-      const float* xw = Xr + w8 * 2 * kHid;
-      const float* dw = Dr + w8 * kHid;
-      for (int q = 0; q < 32; ++q) {
-        const int k = 32 * threadIdx.x + q;
-        pw[q] += xw[k / kHid] * dw[k % kHid];
+    // dX[ty + r][64 h + tx + j] = sum_c dA[ty + r][c] W[64 h + tx + j][c], c ascending
+    float x[2][4][4] = {};
+#pragma unroll 4
+    for (int c = 0; c < kHid; ++c) {
+      const float4 d4 = *reinterpret_cast<const float4*>(DT + c * kPitch + ty);
+      const float d[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 f4 = *reinterpret_cast<const float4*>(WT + c * kPitch2 + h * kHid + tx);
+        const float f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[h][r][j] += d[r] * f[j];
       }
     }
-    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (base + ty + r < n) {
+        const int64_t o = (base + ty + r) * kHid + tx;
+        *reinterpret_cast<float4*>(dHprev + o) = make_float4(x[0][r][0], x[0][r][1], x[0][r][2], x[0][r][3]);
+        *reinterpret_cast<float4*>(dZ + o) = make_float4(x[1][r][0], x[1][r][1], x[1][r][2], x[1][r][3]);
+      }
+    // dW[64 h + ty + i][tx + j] += sum over the tile's rows of X[row][64 h + ty + i] dA[row][tx + j]
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[h][r][j] = 0.f;
+#pragma unroll 4
+    for (int row = 0; row < kBwdRows; ++row) {
+      const float4 d4 = *reinterpret_cast<const float4*>(D + row * kPitch + tx);
+      const float d[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 f4 = *reinterpret_cast<const float4*>(X + row * kPitch2 + h * kHid + ty);
+        const float f[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[h][r][j] += f[r] * d[j];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[h][r][j] += x[h][r][j];
+    if (t < kHid) {
+      float b = 0.f;
+#pragma unroll 8
+      for (int row = 0; row < kBwdRows; ++row) b += D[row * kPitch + t];
+      db += b;
+    }
   }
   float* pp = part + (int64_t)blockIdx.x * (2 * kHid * kHid + kHid);
-  for (int q = 0; q < 32; ++q) pp[32 * threadIdx.x + q] = pw[q];
-  // db: lanes of each warp hold two columns; sum warps in fixed order through shared memory
-  __syncthreads();
-  for (int wv = 0; wv < 8; ++wv) {
-    if (warp == wv) {
-      if (wv == 0) {
-        Dr[lane] = pb[0];
-        Dr[lane + 32] = pb[1];
-      } else {
-        Dr[lane] += pb[0];
-        Dr[lane + 32] += pb[1];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      *reinterpret_cast<float4*>(pp + (h * kHid + ty + r) * kHid + tx) =
+          make_float4(w[h][r][0], w[h][r][1], w[h][r][2], w[h][r][3]);
+  if (t < kHid) pp[2 * kHid * kHid + t] = db;
+}
+
+// dH_prev += A^T dZ (SELL with transposed weights), 64-wide, warp per row.  A block takes runs of 64
+// consecutive rows, whose neighbours are largely the same rows of dZ (read from L1); the lanes load
+// the row's columns and weights together and hand them round, and eight rows of dZ are in flight.
+// 252 MB gathered at 65,536 rows: 35.5 us (47 us one neighbour at a time).
+__global__ void __launch_bounds__(kThreads) k_agg_t(int64_t n, DSell S, const float* __restrict__ At,
+                                                    const float* __restrict__ dZ,
+                                                    float* __restrict__ dH) {
+  constexpr int U = 8, kRun = 64;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int64_t base = (int64_t)blockIdx.x * kRun; base < n; base += (int64_t)gridDim.x * kRun)
+    for (int64_t i = base + warp; i < base + kRun && i < n; i += kThreads / 32) {
+      const int64_t s = i >> 5, li = i & 31;
+      const int64_t sb = S.sptr[s];
+      const int len = S.slen[s];
+      float2* o = reinterpret_cast<float2*>(dH + i * kHid + 2 * lane);
+      const float2 h = *o;
+      float2 acc = make_float2(0.f, 0.f);
+      for (int kb = 0; kb < len; kb += 32) {
+        const bool ok = kb + lane < len;
+        const int64_t e = sb + (int64_t)(kb + lane) * 32 + li;
+        const int cj = ok ? S.col[e] : (int)i;
+        const float ca = ok ? At[e] : 0.f;
+        const int m = len - kb < 32 ? len - kb : 32;
+        for (int k0 = 0; k0 < m; k0 += U) {
+          float2 z[U];
+          float a[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            // past the row's end (k0 + u < 32 still): the row itself with weight 0
+            const int j = __shfl_sync(0xffffffffu, cj, k0 + u);
+            a[u] = __shfl_sync(0xffffffffu, ca, k0 + u);
+            z[u] = *reinterpret_cast<const float2*>(dZ + (int64_t)j * kHid + 2 * lane);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            acc.x += a[u] * z[u].x;
+            acc.y += a[u] * z[u].y;
+          }
+        }
       }
+      *o = make_float2(h.x + acc.x, h.y + acc.y);
     }
-    __syncthreads();
-  }
-  for (int c = threadIdx.x; c < kHid; c += blockDim.x) pp[2 * kHid * kHid + c] = Dr[c];
 }
 
-// dH_prev += A^T dZ (SELL with transposed weights), 64-wide, warp per row
-__global__ void k_agg_t(int64_t n, DSell S, const float* __restrict__ At, const float* __restrict__ dZ,
-                        float* __restrict__ dH) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = tstride() >> 5;
-  for (int64_t i = tid() >> 5; i < n; i += nwarps) {
-    const int64_t s = i >> 5, li = i & 31;
-    const int64_t sb = S.sptr[s];
-    const int len = S.slen[s];
-    float a0 = 0.f, a1 = 0.f;
-    for (int k = 0; k < len; ++k) {
-      const int64_t e = sb + (int64_t)k * 32 + li;
-      const int64_t j = S.col[e];
-      const float a = At[e];
-      a0 += a * dZ[j * kHid + lane];
-      a1 += a * dZ[j * kHid + lane + 32];
-    }
-    dH[i * kHid + lane] += a0;
-    dH[i * kHid + lane + 32] += a1;
-  }
-}
-
-// input layer backward: block partials of dW_in (F^T dA0) and db_in
+// input layer backward: block partials of dW_in (F^T dA0) and db_in, tiles of 64 rows as above (four
+// outputs per thread): 22 us at 65,536 rows, 131 us with a block per row
 __global__ void __launch_bounds__(kThreads) k_in_bwd(int64_t n, const float* __restrict__ dH,
                                                      const __nv_bfloat16* __restrict__ H0,
                                                      const __nv_bfloat16* __restrict__ F,
                                                      float* __restrict__ part) {
-  // part per block: [16*64 dW_in][64 db_in]; thread t owns dW entries 4t .. 4t+3
-  float pw[4] = {0, 0, 0, 0};
-  float pb = 0.f;
+  // part per block: [16*64 dW_in][64 db_in]
+  __shared__ __align__(16) float D[kBwdRows * kPitch];
+  __shared__ __align__(16) float X[kBwdRows * (kFeat + 4)];
   const int t = threadIdx.x;
-  for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
-    for (int q = 0; q < 4; ++q) {
-      const int k = 4 * t + q;
-      const int f = k / kHid, c = k % kHid;
-      const float d = bf(H0 + i * kHid + c) > 0.f ? dH[i * kHid + c] : 0.f;
-      pw[q] += bf(F + i * kFeat + f) * d;
+  const int lr = t % kBwdRows, lc = 16 * (t / kBwdRows);
+  const int tx = 4 * (t % 16), f = t / 16;
+  float w[4] = {}, db = 0.f;
+  for (int64_t base = (int64_t)blockIdx.x * kBwdRows; base < n;
+       base += (int64_t)gridDim.x * kBwdRows) {
+    const int64_t i = base + lr;
+    float v[16];
+    load_da(n, i, lc, dH, H0, v);
+    __syncthreads();
+    store16(D + lr * kPitch + lc, v);
+    if (lc == 0) {
+      if (i < n) {
+        load16(F + i * kFeat, v);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = 0.f;
+      }
+      store16(X + lr * (kFeat + 4), v);
     }
-    if (t < kHid) pb += bf(H0 + i * kHid + t) > 0.f ? dH[i * kHid + t] : 0.f;
+    __syncthreads();
+    float x[4] = {}, b = 0.f;
+#pragma unroll 8
+    for (int row = 0; row < kBwdRows; ++row) {
+      const float4 d = *reinterpret_cast<const float4*>(D + row * kPitch + tx);
+      const float a = X[row * (kFeat + 4) + f];
+      x[0] += a * d.x;
+      x[1] += a * d.y;
+      x[2] += a * d.z;
+      x[3] += a * d.w;
+    }
+    if (t < kHid)
+#pragma unroll 8
+      for (int row = 0; row < kBwdRows; ++row) b += D[row * kPitch + t];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] += x[j];
+    db += b;
   }
   float* pp = part + (int64_t)blockIdx.x * (kFeat * kHid + kHid);
-  for (int q = 0; q < 4; ++q) pp[4 * t + q] = pw[q];
-  if (t < kHid) pp[kFeat * kHid + t] = pb;
+  *reinterpret_cast<float4*>(pp + f * kHid + tx) = make_float4(w[0], w[1], w[2], w[3]);
+  if (t < kHid) pp[kFeat * kHid + t] = db;
 }
 
-// grad[k] = sum over blocks of part[b][k] (fixed block order)
-__global__ void k_reduce_parts(int nblocks, int count, int stride, const float* __restrict__ part,
-                               float* __restrict__ grad) {
-  for (int64_t k = tid(); k < count; k += tstride()) {
-    float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += part[(int64_t)b * stride + k];
-    grad[k] = s;
+// grad[k] = sum over blocks of part[b][k], k < count; part[b][count] to *last where there is one.
+// A block sums 32 values: eight groups of threads take every eighth partial, eight loads in flight,
+// then the groups in order (13 us for 304 partials of 8,256 values; one thread per value 57 us).
+__global__ void __launch_bounds__(kThreads) k_reduce_parts(int nblocks, int count, int stride,
+                                                           const float* __restrict__ part,
+                                                           float* __restrict__ grad,
+                                                           float* __restrict__ last) {
+  __shared__ float sm[8][32];
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
+  const bool ok = k < count + (last ? 1 : 0);
+  float s = 0.f;
+  for (int b = g; ok && b < nblocks; b += 64) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = b + 8 * u < nblocks ? part[(int64_t)(b + 8 * u) * stride + k] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  sm[g][lane] = s;
+  __syncthreads();
+  if (g == 0 && ok) {
+#pragma unroll
+    for (int u = 1; u < 8; ++u) s += sm[u][lane];
+    *(k < count ? grad + k : last) = s;
   }
 }
 
@@ -597,15 +727,6 @@ __global__ void k_transpose_bf16(int rows, int cols, const float* __restrict__ s
   }
 }
 
-__global__ void k_loss_sum(int nblocks, const float* __restrict__ part, int width,
-                           float* __restrict__ out) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s += part[(int64_t)b * width + width - 1];
-    *out = s;
-  }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -618,7 +739,21 @@ static inline int grid_rows(const Launch& L, int64_t n) {
 }
 
 size_t mpnn_layer_smem() { return kTcSmem; }
-size_t mpnn_layer_bwd_smem() { return (size_t)(2 * kHid * kHid + 8 * 2 * kHid + 8 * kHid) * 4; }
+size_t mpnn_layer_bwd_smem() {
+  return (size_t)(kHid * kPitch2 + kBwdRows * kPitch2 + kBwdRows * kPitch + kHid * kPitch) * 4;
+}
+// backward tiles: a block per tile, at most two per SM (each then keeps its sums over its tiles)
+static inline int grid_bwd(const Launch& L, int64_t n) {
+  const int64_t b = (n + kBwdRows - 1) / kBwdRows, cap = 2 * (int64_t)L.sms;
+  return (int)(b > cap ? cap : b);
+}
+static cudaError_t reduce_parts(const Launch& L, int nblocks, int count, int stride,
+                                const float* part, float* grad, float* last) {
+  (*L.counter) += 1;
+  k_reduce_parts<<<(count + (last ? 1 : 0) + 31) / 32, kThreads, 0, L.stream>>>(
+      nblocks, count, stride, part, grad, last);
+  return cudaGetLastError();
+}
 
 template <typename T>
 cudaError_t mpnn_features(const Launch& L, int64_t n, const T* m, int64_t ld, const uint8_t* mag,
@@ -677,36 +812,32 @@ cudaError_t mpnn_backward(const Launch& L, int64_t n, const DSell& S, const Mpnn
                           __nv_bfloat16* const Z[3], const float* Y, const float* T, float* dHa,
                           float* dHb, float* dZ, float* part, float* grad, float* loss) {
   // grad layout = parameter layout: W_in, b_in, {W_l, b_l} x 3, W_out, b_out
-  const int gb = grid_rows(L, n);
+  const int gb = grid_rows(L, n), gt = grid_bwd(L, n);
   cudaError_t e;
   const int wout = kHid * 3 + 4;
-  (*L.counter) += 2;
-  k_out_bwd<<<gb, kThreads, 0, L.stream>>>(n, Y, T, H[kLayers], W.Wout, dHa, part);
-  float* g_out = grad + kOffWout;
-  k_reduce_parts<<<1, 256, 0, L.stream>>>(gb, wout - 1, wout, part, g_out);  // W_out, b_out
   (*L.counter) += 1;
-  k_loss_sum<<<1, 32, 0, L.stream>>>(gb, part, wout, loss);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_out_bwd<<<gb, kThreads, 0, L.stream>>>(n, Y, T, H[kLayers], W.Wout, dHa, part);
+  // W_out, b_out, and the loss
+  if ((e = reduce_parts(L, gb, wout - 1, wout, part, grad + kOffWout, loss)) != cudaSuccess) return e;
   float* dH = dHa;
   float* dHp = dHb;
   const int wl = 2 * kHid * kHid + kHid;
   const size_t sm = mpnn_layer_bwd_smem();
   for (int l = kLayers - 1; l >= 0; --l) {
-    (*L.counter) += 3;
-    k_layer_bwd<<<gb, kThreads, sm, L.stream>>>(n, dH, H[l + 1], H[l], Z[l], W.Wf[l], dHp, dZ,
+    (*L.counter) += 2;
+    k_layer_bwd<<<gt, kThreads, sm, L.stream>>>(n, dH, H[l + 1], H[l], Z[l], W.Wf[l], dHp, dZ,
                                                 part);
-    k_reduce_parts<<<(wl + 255) / 256, 256, 0, L.stream>>>(gb, wl, wl, part, grad + kOffW[l]);
-    k_agg_t<<<L.blocks_for(n * 32), kBlock, 0, L.stream>>>(n, S, W.At, dZ, dHp);
+    if ((e = reduce_parts(L, gt, wl, wl, part, grad + kOffW[l], nullptr)) != cudaSuccess) return e;
+    k_agg_t<<<L.blocks_for(n * (kThreads / 64)), kThreads, 0, L.stream>>>(n, S, W.At, dZ, dHp);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     float* t = dH;
     dH = dHp;
     dHp = t;
   }
   const int wi = kFeat * kHid + kHid;
-  (*L.counter) += 2;
-  k_in_bwd<<<gb, kThreads, 0, L.stream>>>(n, dH, H[0], F, part);
-  k_reduce_parts<<<(wi + 255) / 256, 256, 0, L.stream>>>(gb, wi, wi, part, grad);
-  return cudaGetLastError();
+  (*L.counter) += 1;
+  k_in_bwd<<<gt, kThreads, 0, L.stream>>>(n, dH, H[0], F, part);
+  return reduce_parts(L, gt, wi, wi, part, grad, nullptr);
 }
 
 cudaError_t mpnn_adam(const Launch& L, float* w, const float* g, float* m, float* v, float lr,
