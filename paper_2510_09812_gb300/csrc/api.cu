@@ -1407,11 +1407,28 @@ class Engine final : public EngineBase {
       TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_loop<T>(L_, a, B, 1, npc));
       return GSPM_OK;
     }
-    if (pc) ST(precondition(p_, 1));
-    // singular system: p0 projected off the constants
-    if (!pinned_) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
+    // aggregates that are runs of rows: z is never stored (see launch_pcg_update)
+    const bool runs = pc && pieces_ok_;
+    auto coarse = [&](int first) -> int {
+      TK(GSPM_KCLASS_CG_VEC, launch_pcg_update<T>(L_, SG_, PP_, epr, r_, q_, dinv, pieces_, st, na, first, red_));
+      TK(GSPM_KCLASS_CG_VEC, launch_pcg_coarse<T>(L_, SG_, CC_, PP_, TL, epr == 3 ? crows3_ : crows1_, epr, cinv, rco, pieces_, rc_, qsym_, ec_, st, first, red_));
+      return GSPM_OK;
+    };
+    if (runs) {
+      ST(coarse(1));
+      TK(GSPM_KCLASS_CG_VEC, launch_pcg_p<T>(L_, SG_, CC_, epr, r_, dinv, ec_, p_, x, st, LoopCtl{}, 1));
+    } else {
+      if (pc) ST(precondition(p_, 1));
+      // singular system: p0 projected off the constants
+      if (!pinned_) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
+    }
     auto iter = [&]() -> int {
       TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_spmv<T>(L_, A_, SG_, val, B, 1, len, p_, q_, st, red_, B == 1 ? var_scalar_ : var_block_, pinned_, 1));
+      if (runs) {
+        ST(coarse(0));
+        TK(GSPM_KCLASS_CG_VEC, launch_pcg_p<T>(L_, SG_, CC_, epr, r_, dinv, ec_, p_, x, st, loop_, 0));
+        return GSPM_OK;
+      }
       TK(GSPM_KCLASS_CG_VEC, launch_cg_update<T>(L_, SG_, epr, 1, len, x, r_, p_, q_, st, na, red_));
       if (pc) {
         // z into q (free after the update), then p = z + beta p
@@ -1423,7 +1440,7 @@ class Engine final : public EngineBase {
       return GSPM_OK;
     };
     if (capturing_)
-      ST(cg_graph_loop(slot, iter, B == 1 ? 0 : 1, pc ? 7 : 3));
+      ST(cg_graph_loop(slot, iter, B == 1 ? 0 : 1, runs ? 6 : (pc ? 7 : 3)));
     else
       ST(cg_loop(slot, iter, info));
     // singular system: move the solution to the pinned one (zero at the pinned node)
@@ -1823,6 +1840,57 @@ class Engine final : public EngineBase {
         }
     CC_ = DCoarse{na, d_aor, d_aptr, d_arows, d_aseg, d_agg0, contig};
     pc_ = true;
+    return contig ? init_pieces(aor, agg0) : GSPM_OK;
+  }
+
+  // Pieces of the aggregates in the update's work items, and work items over the coarse rows
+  int init_pieces(const std::vector<int32_t>& aor, const std::vector<int32_t>& agg0) {
+    const int S = nseg_, lst = pcg_resident<T>() - 1;
+    const int ni = SG_.list[lst].nitems;
+    std::vector<int32_t> sl0(ni), sl1(ni), iseg(ni), ip0, prow, ap(agg0[S] + 1, 0);
+    CK(cudaMemcpy(sl0.data(), SG_.list[lst].sl0, ni * 4, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(sl1.data(), SG_.list[lst].sl1, ni * 4, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(iseg.data(), SG_.list[lst].seg, ni * 4, cudaMemcpyDeviceToHost));
+    int max_item = 0;
+    int32_t last = -1;
+    for (int i = 0; i < ni; ++i) {
+      ip0.push_back((int32_t)prow.size());
+      const int64_t r0 = (int64_t)sl0[i] * 32;
+      const int64_t r1 = std::min<int64_t>((int64_t)sl1[i] * 32,
+                                           hb_.seg_row0[iseg[i]] + hb_.seg_nrow[iseg[i]]);
+      for (int64_t row = r0; row < r1; ++row) {
+        const int32_t I = aor[row];
+        if (I != last && I != last + 1) return GSPM_OK;  // not numbered in row order
+        if (I == last && row > r0) continue;
+        prow.push_back((int32_t)row);
+        ++ap[I + 1];
+        last = I;
+      }
+      max_item = std::max(max_item, (int)prow.size() - ip0.back());
+    }
+    ip0.push_back((int32_t)prow.size());
+    for (size_t I = 1; I < ap.size(); ++I) ap[I] += ap[I - 1];
+    // the pieces' slots of a block stay within the 48 KB that need no opt-in
+    if ((size_t)max_item * (kBlock / 32) * 3 * sizeof(T) > 40960) return GSPM_OK;
+    int32_t *d_ip0, *d_row, *d_ap;
+    ST(mem_.alloc(&d_ip0, (int64_t)ip0.size()));
+    ST(mem_.alloc(&d_row, (int64_t)prow.size()));
+    ST(mem_.alloc(&d_ap, (int64_t)ap.size()));
+    ST(mem_.alloc(&pieces_, 3 * (int64_t)prow.size()));
+    CK(cudaMemcpy(d_ip0, ip0.data(), ip0.size() * 4, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(d_row, prow.data(), prow.size() * 4, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(d_ap, ap.data(), ap.size() * 4, cudaMemcpyHostToDevice));
+    PP_ = DPieces{(int)prow.size(), max_item, lst, d_ip0, d_row, d_ap};
+    for (int e = 1; e <= 3; e += 2) {
+      std::vector<int64_t> u0(S), nu(S);
+      for (int sg = 0; sg < S; ++sg) {
+        u0[sg] = (int64_t)e * agg0[sg];
+        nu[sg] = (int64_t)e * (agg0[sg + 1] - agg0[sg]);
+      }
+      int max_items = 0;  // (the reduction scratch holds any list of nseg_ segments)
+      ST(make_item_lists(u0, nu, e == 3 ? crows3_ : crows1_, &max_items));
+    }
+    pieces_ok_ = true;
     return GSPM_OK;
   }
 
@@ -1934,6 +2002,8 @@ class Engine final : public EngineBase {
     item_slices_ = (int)((nslices_ + g.list[0].nitems - 1) / g.list[0].nitems);
     SG_ = g;
     nitems_ = max_items;
+    // (a list's segments round their shares up: at most k x SMs + S items, whatever the units)
+    max_items = std::max(max_items, kItemLists * L_.sms + S);
     ST(mem_.alloc(&red_.partial, (int64_t)max_items * kRedComp));
     return GSPM_OK;
   }
@@ -2145,6 +2215,11 @@ class Engine final : public EngineBase {
   T *dinv3_ = nullptr, *dinv1_ = nullptr;
   T *dgs_eps_ = nullptr, *dgs_aeps_ = nullptr;  // Jacobi of the GSPM solves (NULL: plain)
   T *rc_ = nullptr, *ec_ = nullptr;
+  // two-level CG on aggregates that are runs of rows
+  DPieces PP_{};
+  ItemList crows3_[kItemLists], crows1_[kItemLists];
+  T* pieces_ = nullptr;
+  bool pieces_ok_ = false;
   // volume averages in ABI order
   double *w_abi_ = nullptr, *avg_part_ = nullptr, *host_avg_ = nullptr;
   int64_t *avg_node0_ = nullptr, *avg_count_ = nullptr, avg_max_ = 0;

@@ -140,6 +140,7 @@ __device__ __forceinline__ void cg_start(CGState* st, int* nactive, int nr, cons
   st->zero_x = allow_zero_x ? zero : 0;
   st->pc = pc;
   st->proj = 0;
+  st->xpend = 0;
   for (int a = 0; a < 3; ++a) st->sr[a] = st->sub[a] = 0.0;
   if (any) atomicAdd(nactive, 1);
 }
@@ -367,7 +368,10 @@ __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_cg_spmv(DSell A, 
   for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
     const int seg = IL.seg[item];
     CGState* sg = st + seg;
-    if (!sg->active) continue;
+    if (!sg->active) {
+      if (threadIdx.x == 0) sg->xpend = 0;  // (every block of the segment, the same value)
+      continue;
+    }
     const int64_t pin = pinned ? G.seg_pin[seg] : -1;
     int skip[NR];
 #pragma unroll
@@ -423,6 +427,7 @@ __global__ void __launch_bounds__(kBlock, min_blocks<VAR>()) k_cg_spmv(DSell A, 
         CGRhs& c = sg->r[k];
         if (c.done) continue;
         c.pq = res[k];
+        sg->xpend = res[k] > 0.0;
         if (res[k] > 0.0) {
           c.alpha = (sg->pc ? c.rz : c.rr) / res[k];
         } else {  // p = 0: nothing left to reduce
@@ -761,82 +766,6 @@ __global__ void __launch_bounds__(kBlock) k_restrict(DCoarse C, const T* __restr
 }
 
 
-// The same for contiguous aggregates (GSPM_ORDER_AGGREGATE) of scalar rows: one warp per
-// aggregate, no barrier.  The aggregate's elements [e0, e1) of r are read as 16-byte packs, kRestrictPacks per
-// lane in flight, with the unaligned head and tail (fewer than one pack each) taken by single
-// lanes; element e has component e mod EPR.  Each lane sums its packs in order, the warp tree is
-// fixed, so the result does not depend on the grid.
-constexpr int kRestrictPacks = 8;
-template <typename T, int EPR>
-__global__ void __launch_bounds__(kBlock) k_restrict_contig(DCoarse C, const T* __restrict__ r,
-                                                            const int64_t* __restrict__ rc_off,
-                                                            T* __restrict__ rc) {
-  pdl_enter();
-  constexpr int W = Pack16<T>::W, U = kRestrictPacks;
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t I = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; I < C.nagg;
-       I += nwarps) {
-    const int q0 = C.agg_ptr[I], q1 = C.agg_ptr[I + 1];
-    T acc[EPR];
-#pragma unroll
-    for (int a = 0; a < EPR; ++a) acc[a] = T(0);
-    if (q1 > q0) {
-      const int64_t e0 = (int64_t)C.agg_rows[q0] * EPR, e1 = e0 + (int64_t)(q1 - q0) * EPR;
-      int64_t a0 = (e0 + W - 1) / W * W;
-      if (a0 > e1) a0 = e1;
-      int64_t a1 = e1 / W * W;
-      if (a1 < a0) a1 = a0;
-      const int nh = (int)(a0 - e0), nt = (int)(e1 - a1);
-      if (lane < nh + nt) {
-        const int64_t e = lane < nh ? e0 + lane : a1 + (lane - nh);
-        acc[EPR == 1 ? 0 : (int)(e % EPR)] += r[e];
-      }
-      const int64_t np = (a1 - a0) / W;
-      const int cb0 = EPR == 1 ? 0 : (int)(a0 % EPR);
-      for (int64_t t0 = 0; t0 < np; t0 += 32 * U) {
-        T v[U][W];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int64_t t = t0 + 32 * u + lane;
-          if (t < np) {
-            ld16(r + a0 + t * W, v[u]);
-          } else {
-#pragma unroll
-            for (int c = 0; c < W; ++c) v[u][c] = T(0);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int64_t t = t0 + 32 * u + lane;
-          // component of the pack's first element: (a0 + t W) mod EPR
-          const int cb = EPR == 1 ? 0 : (int)((cb0 + (t % EPR) * (W % EPR)) % EPR);
-#pragma unroll
-          for (int c = 0; c < W; ++c) {
-            if (EPR == 1) {
-              acc[0] += v[u][c];
-            } else {
-              const int cc = (cb + c) % EPR;
-#pragma unroll
-              for (int a = 0; a < EPR; ++a) acc[a] += cc == a ? v[u][c] : T(0);
-            }
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < EPR; ++a) {
-      T v = acc[a];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-      if (lane == 0) {
-        const int sg = C.agg_seg[I];
-        rc[rc_off[sg] + (I - C.seg_agg0[sg]) * EPR + a] = v;
-      }
-    }
-  }
-}
-
 // N contiguous values through 16-byte packs (N * sizeof(T) a multiple of 16, p aligned)
 template <typename T, int N>
 __device__ __forceinline__ void ldn(const T* p, T (&v)[N]) {
@@ -1072,6 +1001,319 @@ __global__ void __launch_bounds__(kBlock) k_pcg_z(DSeg G, ItemList IL, DCoarse C
   }
 }
 
+
+// ------------------------------------------------------------------------------------------
+// two-level CG with z never stored (aggregates that are runs of rows)
+// ------------------------------------------------------------------------------------------
+// Bound by HBM above the L2's size.  Vector traffic per iteration in vectors of n values: update 4
+// (r in and out, q, D^-1), p-update 6 (r, D^-1, p and x in and out); the update, restriction, z and
+// p-update kernels moved 15 (x, r and p, q, then r, then r, D^-1 and z, then z and p).  The p-update
+// takes x along because it reads p anyway.  A step of 2,963,088 nodes (two of 548 two-level
+// iterations): 217.3 -> 213.5 ms; 16 meshes of 65,536 nodes: 43.2 -> 41.6 ms.
+//
+// Four rows per thread and round (whole 16-byte packs: item ranges start at multiples of 32 rows).
+// A warp's 128 rows lie in one or two aggregates: it sums each by shuffles into its own slot of the
+// piece, and the block's eight slots are added at the end (no barrier per aggregate).
+template <typename T, int EPR>
+__global__ void __launch_bounds__(kBlock, pcg_resident<T>())
+    k_pcg_update(DSeg G, ItemList IL, DPieces PP, T* __restrict__ r, const T* __restrict__ q,
+                 const T* __restrict__ dinv, T* __restrict__ pieces, CGState* st, int* nactive,
+                 int first, Red red) {
+  pdl_enter();
+  constexpr int N = 4 * EPR, NW = kBlock / 32;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  T* ps = reinterpret_cast<T*>(dyn);  // [piece of the item][warp][EPR]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
+    const int seg = IL.seg[item];
+    CGState* sg = st + seg;
+    if (!sg->active) continue;
+    const bool proj = sg->proj;
+    const T al = first || sg->r[0].done ? T(0) : (T)sg->r[0].alpha;
+    const bool upd = !first && !sg->r[0].done;
+    const int64_t r0 = (int64_t)IL.sl0[item] * 32;
+    const int64_t rend = G.seg_row0[seg] + G.seg_nrow[seg];
+    const int64_t rhi = (int64_t)IL.sl1[item] * 32;
+    const int64_t r1 = rhi < rend ? rhi : rend;
+    const int p0 = PP.item_p0[item], np = PP.item_p0[item + 1] - p0;
+    for (int k = threadIdx.x; k < np * NW * EPR; k += kBlock) ps[k] = T(0);
+    __syncthreads();
+    // r.r, r.D^-1 r (compensated), sums of r and of D^-1 r
+    T rr = T(0), dz = T(0), dzc = T(0), sr[EPR], sd[EPR];
+#pragma unroll
+    for (int a = 0; a < EPR; ++a) sr[a] = sd[a] = T(0);
+    int pc = 0;
+    for (int64_t w0 = r0 + 128 * warp; w0 < r1; w0 += 128 * NW) {
+      const int64_t row = w0 + 4 * lane;
+      T rv[N];
+#pragma unroll
+      for (int e = 0; e < N; ++e) rv[e] = T(0);
+      if (row + 4 <= r1) {
+        T dv[N];
+        ldn<T, N>(r + row * EPR, rv);
+        ldn<T, N>(dinv + row * EPR, dv);
+        if (upd) {
+          T qv[N];
+          ldn<T, N>(q + row * EPR, qv);
+#pragma unroll
+          for (int e = 0; e < N; ++e) rv[e] -= al * qv[e];
+          stn<T, N>(r + row * EPR, rv);
+        }
+        T t = T(0);
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+          const T z = dv[e] * rv[e];
+          rr += rv[e] * rv[e];
+          t += rv[e] * z;
+          sr[e % EPR] += rv[e];
+          sd[e % EPR] += z;
+        }
+        kahan_add(dz, dzc, t);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (row + u < r1) {
+#pragma unroll
+            for (int a = 0; a < EPR; ++a) {
+              const int64_t e = (row + u) * EPR + a;
+              T v = r[e];
+              if (upd) {
+                v -= al * q[e];
+                r[e] = v;
+              }
+              const T z = dinv[e] * v;
+              rr += v * v;
+              kahan_add(dz, dzc, v * z);
+              sr[a] += v;
+              sd[a] += z;
+              rv[u * EPR + a] = v;
+            }
+          }
+      }
+      // pieces of the warp's rows
+      while (pc + 1 < np && PP.row[p0 + pc + 1] <= w0) ++pc;
+      for (int k = pc; k < np; ++k) {
+        const int64_t b = PP.row[p0 + k];
+        if (b >= w0 + 128) break;
+        const int64_t e = k + 1 < np ? (int64_t)PP.row[p0 + k + 1] : r1;
+        T v[EPR];
+#pragma unroll
+        for (int a = 0; a < EPR; ++a) v[a] = T(0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (row + u >= b && row + u < e)
+#pragma unroll
+            for (int a = 0; a < EPR; ++a) v[a] += rv[u * EPR + a];
+#pragma unroll
+        for (int a = 0; a < EPR; ++a) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v[a] += __shfl_down_sync(kFull, v[a], o);
+          if (lane == 0) ps[(k * NW + warp) * EPR + a] += v[a];
+        }
+      }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < np * EPR; k += kBlock) {
+      T v = T(0);
+#pragma unroll
+      for (int w = 0; w < NW; ++w) v += ps[((k / EPR) * NW + w) * EPR + k % EPR];
+      pieces[(int64_t)p0 * EPR + k] = v;
+    }
+    T hi[2 + 2 * EPR], lo[2 + 2 * EPR];
+#pragma unroll
+    for (int v = 0; v < 2 + 2 * EPR; ++v) lo[v] = T(0);
+    hi[0] = rr;
+    hi[1] = dz;
+    lo[1] = -dzc;
+#pragma unroll
+    for (int a = 0; a < EPR; ++a) {
+      hi[2 + a] = sr[a];
+      hi[2 + EPR + a] = sd[a];
+    }
+    __shared__ double res[2 + 2 * EPR];
+    if (seg_reduce_hl<T, 2 + 2 * EPR>(hi, lo, item, seg, G, IL, red, res) && threadIdx.x == 0) {
+      CGRhs& c = sg->r[0];
+      sg->rdr = res[1];
+      for (int a = 0; a < EPR; ++a) sg->sd[a] = res[2 + EPR + a];
+      if (!first) {
+        int any = 0;
+        if (!c.done) {
+          c.iters += 1;
+          double rrk = res[0];
+          if (proj) {
+            // r.r without r's constant part
+            double s2 = 0.0;
+            for (int a = 0; a < EPR; ++a) {
+              sg->sr[a] = res[2 + a];
+              s2 += res[2 + a] * res[2 + a];
+            }
+            rrk -= s2 / (double)G.seg_nrow[seg];
+            rrk = rrk > 0.0 ? rrk : 0.0;
+          }
+          c.rr = rrk;
+          if (rrk < c.tol2) {
+            c.done = 1;
+          } else if (c.iters >= sg->max_iter) {
+            c.done = 1;
+            sg->noconv += 1;
+          }
+          any = !c.done;
+        }
+        sg->active = any;
+        if (!any) atomicSub(nactive, 1);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// rc(I, a) = sum of aggregate I's pieces, in row order
+template <typename T, int EPR>
+__global__ void __launch_bounds__(kBlock) k_piece_sum(DCoarse C, DPieces PP,
+                                                      const T* __restrict__ pieces,
+                                                      const int64_t* __restrict__ rc_off,
+                                                      T* __restrict__ rc) {
+  pdl_enter();
+  for (int64_t g = gtid(); g < C.nagg * EPR; g += gstride()) {
+    const int I = (int)(g / EPR), a = (int)(g % EPR), sg = C.agg_seg[I];
+    T v = T(0);
+    for (int k = PP.ap[I]; k < PP.ap[I + 1]; ++k) v += pieces[(int64_t)k * EPR + a];
+    rc[rc_off[sg] + (I - C.seg_agg0[sg]) * EPR + a] = v;
+  }
+}
+
+// ec(g) = the sum of row g of Q (one warp per coarse row, lanes over the columns, fixed order), and
+// per segment r_c.e_c and the sums over its rows of P e_c: with the update's sums they give r.z and
+// the mean of z, hence beta
+template <typename T, int EPR>
+__global__ void __launch_bounds__(kBlock) k_pcg_coarse(DSeg G, ItemList IL, DCoarse C, DSymTiles TL,
+                                                       const T* __restrict__ Q,
+                                                       const int64_t* __restrict__ rc_off,
+                                                       const T* __restrict__ rc, T* __restrict__ ec,
+                                                       CGState* st, int first, Red red) {
+  pdl_enter();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
+    const int seg = IL.seg[item];
+    CGState* sg = st + seg;
+    if (!sg->active) continue;
+    const int64_t g0 = (int64_t)C.seg_agg0[seg] * EPR, Tn = TL.seg_T[seg];
+    T hi[1 + EPR], lo[1 + EPR];
+#pragma unroll
+    for (int v = 0; v < 1 + EPR; ++v) hi[v] = lo[v] = T(0);
+    for (int64_t g = IL.sl0[item] + warp; g < IL.sl1[item]; g += kBlock / 32) {
+      const int64_t loc = g - g0;
+      const T* qr = Q + TL.seg_q0[seg] + loc * Tn;
+      T acc = T(0);
+      for (int64_t j = lane; j < Tn; j += 32) acc += qr[j];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
+      if (lane == 0) {
+        ec[g] = acc;
+        const int I = (int)(g / EPR), a = (int)(g - (int64_t)I * EPR);
+        const T cnt = (T)(C.agg_ptr[I + 1] - C.agg_ptr[I]);
+        kahan_add(hi[0], lo[0], acc * rc[rc_off[seg] + loc]);
+#pragma unroll
+        for (int b = 0; b < EPR; ++b)
+          if (a == b) kahan_add(hi[1 + b], lo[1 + b], cnt * acc);
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 1 + EPR; ++v) lo[v] = -lo[v];
+    __shared__ double res[1 + EPR];
+    if (seg_reduce_hl<T, 1 + EPR>(hi, lo, item, seg, G, IL, red, res) && threadIdx.x == 0) {
+      CGRhs& c = sg->r[0];
+      double rz = sg->rdr + res[0];
+      if (sg->proj) {
+        // z projected off the constants (the p-update subtracts its mean): r.(z - zbar 1)
+        const double inv_n = 1.0 / (double)G.seg_nrow[seg];
+        for (int a = 0; a < EPR; ++a) {
+          const double zbar = (sg->sd[a] + res[1 + a]) * inv_n;
+          rz -= zbar * sg->sr[a];
+          sg->sub[a] = zbar;
+        }
+      }
+      if (!first) c.beta = c.rz != 0.0 ? rz / c.rz : 0.0;
+      c.rz = rz;
+    }
+  }
+}
+
+// x += alpha p (if pending), then p = D^-1 r + P ec - mean + beta p on the active segments; first:
+// p = z - mean.  In a graph loop block 0 also decides whether the loop runs again.
+template <typename T, int EPR>
+__global__ void __launch_bounds__(kBlock) k_pcg_p(DSeg G, ItemList IL, DCoarse C,
+                                                  const T* __restrict__ r,
+                                                  const T* __restrict__ dinv,
+                                                  const T* __restrict__ ec, T* __restrict__ p,
+                                                  T* __restrict__ x, const CGState* st, LoopCtl lc,
+                                                  int first) {
+  pdl_enter();
+  constexpr int N = 4 * EPR;
+  if (lc.count && blockIdx.x == 0 && threadIdx.x == 0) {
+    const int c = *lc.count + 1;
+    *lc.count = c;
+    *lc.total += (unsigned long long)lc.body;
+    cudaGraphSetConditional(lc.handle, (__ldcg(lc.nactive) > 0 && c < lc.limit) ? 1u : 0u);
+  }
+  for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
+    const int seg = IL.seg[item];
+    const CGState* sg = st + seg;
+    const bool xp = !first && sg->xpend, act = sg->active;
+    if (!xp && !act) continue;
+    const T al = (T)sg->r[0].alpha, be = first ? T(0) : (T)sg->r[0].beta;
+    T sb[EPR];
+#pragma unroll
+    for (int a = 0; a < EPR; ++a) sb[a] = sg->proj ? (T)sg->sub[a] : T(0);
+    const int64_t r0 = (int64_t)IL.sl0[item] * 32;
+    const int64_t rend = G.seg_row0[seg] + G.seg_nrow[seg];
+    const int64_t rhi = (int64_t)IL.sl1[item] * 32;
+    const int64_t r1 = rhi < rend ? rhi : rend;
+    const int64_t ng = (r1 - r0) / 4;
+    for (int64_t g = threadIdx.x; g < ng; g += blockDim.x) {
+      const int64_t row = r0 + 4 * g;
+      T pv[N];
+#pragma unroll
+      for (int e = 0; e < N; ++e) pv[e] = T(0);
+      if (!first) ldn<T, N>(p + row * EPR, pv);
+      if (xp) {
+        T xv[N];
+        ldn<T, N>(x + row * EPR, xv);
+#pragma unroll
+        for (int e = 0; e < N; ++e) xv[e] += al * pv[e];
+        stn<T, N>(x + row * EPR, xv);
+      }
+      if (act) {
+        T rv[N], dv[N];
+        ldn<T, N>(r + row * EPR, rv);
+        ldn<T, N>(dinv + row * EPR, dv);
+        const int4 ag = *reinterpret_cast<const int4*>(C.agg_of_row + row);
+        const int agv[4] = {ag.x, ag.y, ag.z, ag.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int a = 0; a < EPR; ++a) {
+            const int e = u * EPR + a;
+            const T z = (dv[e] * rv[e] + ec[(int64_t)agv[u] * EPR + a]) - sb[a];
+            pv[e] = first ? z : z + be * pv[e];
+          }
+        stn<T, N>(p + row * EPR, pv);
+      }
+    }
+    for (int64_t row = r0 + 4 * ng + threadIdx.x; row < r1; row += blockDim.x) {
+      const int64_t I = C.agg_of_row[row];
+#pragma unroll
+      for (int a = 0; a < EPR; ++a) {
+        const int64_t e = row * EPR + a;
+        if (xp) x[e] += al * p[e];
+        if (act) {
+          const T z = (dinv[e] * r[e] + ec[I * EPR + a]) - sb[a];
+          p[e] = first ? z : z + be * p[e];
+        }
+      }
+    }
+  }
+}
 
 __global__ void k_loop_start(LoopCtl lc) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1673,11 +1915,12 @@ static ItemGrid item_grid(const Launch& L, const DSeg& G, const void* kernel) {
 
 // Launch of a CG loop kernel with programmatic stream serialisation (see pdl_enter)
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*k)(KArgs...), int grid, cudaStream_t stream, Args... args) {
+static cudaError_t launch_pdl_smem(void (*k)(KArgs...), int grid, size_t smem, cudaStream_t stream,
+                                   Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kBlock);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1685,6 +1928,10 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), int grid, cudaStream_t stream
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k, args...);
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(void (*k)(KArgs...), int grid, cudaStream_t stream, Args... args) {
+  return launch_pdl_smem(k, grid, 0, stream, args...);
 }
 
 #define GSPM_GRID(L, threads, kern) grid_for((L), (threads), reinterpret_cast<const void*>(kern))
@@ -1975,12 +2222,7 @@ template <typename T>
 cudaError_t launch_restrict(const Launch& L, const DCoarse& C, int epr, const T* r,
                             const int64_t* rc_off, T* rc) {
   (*L.counter) += 1;
-  // scalar rows: a warp per contiguous aggregate (6.4 against 13 us per launch at 3M nodes,
-  // cold); three components: a block per aggregate (15.9 us against 23 us for a warp)
-  if (epr == 1 && C.contig && aligned16(r)) {
-    auto k = k_restrict_contig<T, 1>;
-    ST_CUDA(launch_pdl(k, GSPM_GRID(L, C.nagg * 32, k), L.stream, C, r, rc_off, rc));
-  } else if (epr == 3) {
+  if (epr == 3) {
     auto k = k_restrict<T, 3>;
     ST_CUDA(launch_pdl(k, GSPM_GRID(L, C.nagg * kBlock, k), L.stream, C, r, rc_off, rc));
   } else if (epr == 1) {
@@ -2004,6 +2246,78 @@ cudaError_t launch_coarse_symv(const Launch& L, const DCoarse& C, const DSymTile
   ST_CUDA(launch_pdl(k2, GSPM_GRID(L, C.nagg * epr * 32, k2), L.stream, C, TL, epr, Q, ec));
   return cudaGetLastError();
 }
+template <typename T, int EPR>
+static cudaError_t pcg_update_n(const Launch& L, const DSeg& G, const DPieces& PP, T* r, const T* q,
+                                const T* dinv, T* pieces, CGState* st, int* nactive, int first,
+                                Red red) {
+  auto k = k_pcg_update<T, EPR>;
+  const ItemList& il = G.list[PP.list];
+  const size_t smem = (size_t)PP.max_item * (kBlock / 32) * EPR * sizeof(T);
+  return launch_pdl_smem(k, std::min(il.nitems, L.max_blocks), smem, L.stream, G, il, PP, r, q, dinv,
+                         pieces, st, nactive, first, red);
+}
+
+template <typename T>
+cudaError_t launch_pcg_update(const Launch& L, const DSeg& G, const DPieces& PP, int epr, T* r,
+                              const T* q, const T* dinv, T* pieces, CGState* st, int* nactive,
+                              int first, Red red) {
+  (*L.counter) += 1;
+  if (!aligned16(r) || !aligned16(q) || !aligned16(dinv)) return cudaErrorInvalidValue;
+  return epr == 3 ? pcg_update_n<T, 3>(L, G, PP, r, q, dinv, pieces, st, nactive, first, red)
+                  : pcg_update_n<T, 1>(L, G, PP, r, q, dinv, pieces, st, nactive, first, red);
+}
+
+template <typename T, int EPR>
+static cudaError_t pcg_coarse_n(const Launch& L, const DSeg& G, const DCoarse& C, const DPieces& PP,
+                                const DSymTiles& TL, const ItemList (&crows)[kItemLists],
+                                const typename CoarseStore<T>::type* inv, const int64_t* rc_off,
+                                const T* pieces, T* rc, T* Q, T* ec, CGState* st, int first,
+                                Red red) {
+  auto k0 = k_piece_sum<T, EPR>;
+  ST_CUDA(launch_pdl(k0, GSPM_GRID(L, C.nagg * EPR, k0), L.stream, C, PP, pieces, rc_off, rc));
+  auto k1 = k_coarse_symv_tiles<T, typename CoarseStore<T>::type>;
+  ST_CUDA(launch_pdl(k1, GSPM_GRID(L, TL.ntiles * kBlock, k1), L.stream, TL, inv, rc_off,
+                     (const T*)rc, Q));
+  auto k2 = k_pcg_coarse<T, EPR>;
+  const int per_sm = resident_per_sm(reinterpret_cast<const void*>(k2));
+  const ItemList& il = crows[(per_sm < kItemLists ? per_sm : kItemLists) - 1];
+  return launch_pdl(k2, grid_for(L, (int64_t)il.nitems * kBlock, reinterpret_cast<const void*>(k2)),
+                    L.stream, G, il, C, TL, (const T*)Q, rc_off, (const T*)rc, ec, st, first, red);
+}
+
+template <typename T>
+cudaError_t launch_pcg_coarse(const Launch& L, const DSeg& G, const DCoarse& C, const DPieces& PP,
+                              const DSymTiles& TL, const ItemList (&crows)[kItemLists], int epr,
+                              const typename CoarseStore<T>::type* inv, const int64_t* rc_off,
+                              const T* pieces, T* rc, T* Q, T* ec, CGState* st, int first, Red red) {
+  (*L.counter) += 3;
+  if (!aligned16(inv) || !aligned16(rc)) return cudaErrorInvalidValue;
+  return epr == 3 ? pcg_coarse_n<T, 3>(L, G, C, PP, TL, crows, inv, rc_off, pieces, rc, Q, ec, st,
+                                       first, red)
+                  : pcg_coarse_n<T, 1>(L, G, C, PP, TL, crows, inv, rc_off, pieces, rc, Q, ec, st,
+                                       first, red);
+}
+
+template <typename T, int EPR>
+static cudaError_t pcg_p_n(const Launch& L, const DSeg& G, const DCoarse& C, const T* r,
+                           const T* dinv, const T* ec, T* p, T* x, const CGState* st,
+                           const LoopCtl& lc, int first) {
+  auto k = k_pcg_p<T, EPR>;
+  const ItemGrid ig = GSPM_IGRID(L, G, k);
+  return launch_pdl(k, ig.grid, L.stream, G, ig.list, C, r, dinv, ec, p, x, st, lc, first);
+}
+
+template <typename T>
+cudaError_t launch_pcg_p(const Launch& L, const DSeg& G, const DCoarse& C, int epr, const T* r,
+                         const T* dinv, const T* ec, T* p, T* x, const CGState* st,
+                         const LoopCtl& lc, int first) {
+  (*L.counter) += 1;
+  if (!aligned16(r) || !aligned16(dinv) || !aligned16(p) || !aligned16(x))
+    return cudaErrorInvalidValue;
+  return epr == 3 ? pcg_p_n<T, 3>(L, G, C, r, dinv, ec, p, x, st, lc, first)
+                  : pcg_p_n<T, 1>(L, G, C, r, dinv, ec, p, x, st, lc, first);
+}
+
 template <typename T>
 cudaError_t launch_pcg_z(const Launch& L, const DSeg& G, const DCoarse& C, int epr, const T* r,
                          const T* dinv, const T* ec, T* z, CGState* st, int init, Red red) {
@@ -2220,6 +2534,15 @@ cudaError_t launch_scaled_diff(const Launch& L, int64_t len, const T* a, const T
   template cudaError_t launch_coarse_symv<T>(const Launch&, const DCoarse&, const DSymTiles&, int, \
                                              const typename CoarseStore<T>::type*, const int64_t*, \
                                              const T*, T*, T*);                                   \
+  template cudaError_t launch_pcg_update<T>(const Launch&, const DSeg&, const DPieces&, int, T*,  \
+                                            const T*, const T*, T*, CGState*, int*, int, Red);    \
+  template cudaError_t launch_pcg_coarse<T>(                                                      \
+      const Launch&, const DSeg&, const DCoarse&, const DPieces&, const DSymTiles&,               \
+      const ItemList(&)[kItemLists], int, const typename CoarseStore<T>::type*, const int64_t*,   \
+      const T*, T*, T*, T*, CGState*, int, Red);                                                  \
+  template cudaError_t launch_pcg_p<T>(const Launch&, const DSeg&, const DCoarse&, int, const T*, \
+                                       const T*, const T*, T*, T*, const CGState*,                \
+                                       const LoopCtl&, int);                                      \
   template cudaError_t launch_pcg_z<T>(const Launch&, const DSeg&, const DCoarse&, int, const T*, \
                                        const T*, const T*, T*, CGState*, int, Red);              \
   template cudaError_t launch_cg_init_gs<T>(const Launch&, const DSell&, const DSeg&, const T*,   \

@@ -61,8 +61,10 @@ struct CGState {
   // proj: CG on the singular system projected off the constants (one right-hand side):
   // sr = per-component sums of r, sub = the per-component mean that the p-update subtracts
   // from its input (z, or r without preconditioner)
-  int proj, pad;
+  // xpend: x += alpha p is still to be done (the two-level CG's p-update does it, see k_pcg_p)
+  int proj, xpend;
   double sr[3], sub[3];
+  double rdr, sd[3];  // r.D^-1 r and the sums of D^-1 r of the two-level update
 };
 
 // Aggregates of the two-level preconditioner, all segments: rows of aggregate I are
@@ -242,6 +244,35 @@ template <typename T>
 cudaError_t launch_coarse_symv(const Launch& L, const DCoarse& C, const DSymTiles& TL, int epr,
                                const typename CoarseStore<T>::type* inv, const int64_t* rc_off,
                                const T* rc, T* Q, T* ec);
+// Two-level CG on aggregates that are runs of rows (DCoarse::contig), z never stored: the update
+// forms r, the sums of the residual and of D^-1 r, and the restricted residual piece by piece (a
+// piece: the part of an aggregate in one work item); the coarse product's last step adds r_c.e_c
+// and the sums of P e_c and gives beta; the p-update forms z = D^-1 r + P e_c on the fly.
+struct DPieces {
+  int npieces, max_item;       // all pieces, most pieces of an item
+  int list;                    // the items' list (resident blocks per SM - 1)
+  const int32_t* item_p0;      // [items + 1] first piece of each item
+  const int32_t* row;          // [pieces] first row
+  const int32_t* ap;           // [nagg + 1] first piece of each aggregate
+};
+// blocks per SM that the update is compiled for
+template <typename T>
+constexpr int pcg_resident() { return sizeof(T) == 4 ? 4 : 2; }
+template <typename T>
+cudaError_t launch_pcg_update(const Launch& L, const DSeg& G, const DPieces& PP, int epr, T* r,
+                              const T* q, const T* dinv, T* pieces, CGState* st, int* nactive,
+                              int first, Red red);
+// rc from the pieces, ec = A_c^-1 rc, then rz (first) or beta and rz, and the means for the p-update.
+// crows: work items over the coarse rows.
+template <typename T>
+cudaError_t launch_pcg_coarse(const Launch& L, const DSeg& G, const DCoarse& C, const DPieces& PP,
+                              const DSymTiles& TL, const ItemList (&crows)[kItemLists], int epr,
+                              const typename CoarseStore<T>::type* inv, const int64_t* rc_off,
+                              const T* pieces, T* rc, T* Q, T* ec, CGState* st, int first, Red red);
+template <typename T>
+cudaError_t launch_pcg_p(const Launch& L, const DSeg& G, const DCoarse& C, int epr, const T* r,
+                         const T* dinv, const T* ec, T* p, T* x, const CGState* st,
+                         const LoopCtl& lc, int first);
 template <typename T>
 cudaError_t launch_pcg_z(const Launch& L, const DSeg& G, const DCoarse& C, int epr, const T* r,
                          const T* dinv, const T* ec, T* z, CGState* st, int init, Red red);
