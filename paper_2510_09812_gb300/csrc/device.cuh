@@ -14,12 +14,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-__device__ __forceinline__ double warp_sum(double x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-  return x;
-}
-
 // Compensated summation (Kahan): s + c carries the running sum with the low-order part lost by
 // each add kept in c (subtracted at the end: total = s - c)
 template <typename T>
@@ -42,67 +36,6 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// The last item of `seg` to arrive (its block partials already in red.partial[item]) sums the
-// segment's item partials in item order and returns true (totals in res[0..NC), valid in every
-// thread of that block).
-template <int NC>
-__device__ __forceinline__ bool seg_arrive(int item, int seg, const DSeg& G, const ItemList& IL,
-                                           const Red& red, double* res) {
-  __shared__ double sm[NC][32];
-  __shared__ int am_last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned t = atomicAdd(G.counter + seg, 1u);
-    am_last = (t == (unsigned)IL.seg_nitems[seg] - 1u);
-  }
-  __syncthreads();
-  if (!am_last) return false;
-  __threadfence();
-  const int i0 = IL.seg_item0[seg], ni = IL.seg_nitems[seg];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < ni; b += blockDim.x)
-      acc += __ldcg(red.partial + (int64_t)(i0 + b) * kRedComp + c);
-    acc = warp_sum(acc);
-    if (lane == 0) sm[c][warp] = acc;
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const double x = warp_sum(lane < nw ? sm[c][lane] : 0.0);
-      if (lane == 0) res[c] = x;
-    }
-  }
-  if (threadIdx.x == 0) G.counter[seg] = 0u;
-  __syncthreads();
-  return true;
-}
-
-// Block reduction of NC values into partial[item] (FP64 tree), then seg_arrive.
-template <int NC>
-__device__ __forceinline__ bool seg_reduce(double (&v)[NC], int item, int seg, const DSeg& G,
-                                           const ItemList& IL, const Red& red, double* res) {
-  __shared__ double sm[NC][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    const double x = warp_sum(v[c]);
-    if (lane == 0) sm[c][warp] = x;
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const double x = warp_sum(lane < nw ? sm[c][lane] : 0.0);
-      if (lane == 0) red.partial[(int64_t)item * kRedComp + c] = x;
-    }
-  }
-  return seg_arrive<NC>(item, seg, G, IL, red, res);
-}
-
 // Double-float addition (h, l) += (bh, bl): Knuth's TwoSum of the high parts, the low parts
 // added to its error term, renormalised (the _rn intrinsics keep the compiler from contracting
 // or reassociating the steps)
@@ -113,6 +46,144 @@ __device__ __forceinline__ void df_add(float& h, float& l, float bh, float bl) {
   e = __fadd_rn(e, __fadd_rn(l, bl));
   h = __fadd_rn(s, e);
   l = __fsub_rn(e, __fsub_rn(h, s));
+}
+
+// a double-float value; the three operations that the sums over lanes need, for each type
+struct DF {
+  float h, l;
+};
+__device__ __forceinline__ DF lane_xor(DF v, int o) {
+  return DF{__shfl_xor_sync(kFull, v.h, o), __shfl_xor_sync(kFull, v.l, o)};
+}
+template <typename V>
+__device__ __forceinline__ V lane_xor(V v, int o) {
+  return __shfl_xor_sync(kFull, v, o);
+}
+__device__ __forceinline__ DF plus(DF a, DF b) {
+  df_add(a.h, a.l, b.h, b.l);
+  return a;
+}
+template <typename V>
+__device__ __forceinline__ V plus(V a, V b) {
+  return a + b;
+}
+__device__ __forceinline__ double as_double(DF v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double as_double(double v) { return v; }
+
+__host__ __device__ constexpr int pow2_up(int n) { return n <= 1 ? 1 : 2 * pow2_up((n + 1) / 2); }
+
+// Sums of M values (a power of two) over each group of LANES lanes.  While several values are
+// left, a pair of lanes splits them: each keeps half of them and adds the other lane's, so M
+// values take M - 1 + log2(LANES / M) additions where M separate trees take M log2(LANES).  The
+// result is value (lane % LANES) / (LANES / M), the same bits in every lane that has it.
+template <int M, int LANES, typename V>
+__device__ __forceinline__ V lane_sums(V (&v)[M]) {
+  const int lane = threadIdx.x & 31;
+  int o = LANES / 2;
+#pragma unroll
+  for (int w = M / 2; w >= 1; w >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const V send = up ? v[i] : v[i + w];
+      v[i] = plus(up ? v[i + w] : v[i], lane_xor(send, o));
+    }
+    o >>= 1;
+  }
+#pragma unroll
+  for (int r = LANES / M; r > 1; r >>= 1) v[0] = plus(v[0], lane_xor(v[0], r / 2));
+  return v[0];
+}
+
+// The last item of `seg` to arrive (its block partials, a row of pow2_up(NC) values, already in
+// red.partial) sums the segment's item partials in a fixed order and returns true (totals in
+// res[0..NC), valid in every thread of that block).  The partials of a segment are one run that
+// the whole block loads in order, every load independent of the others; thread t sums value
+// t % pow2_up(NC).  FP64 additions bound this tail (2 per clock and SM): one per partial value,
+// the trees over lanes only as deep as a value has lanes.  Against one strided pass, one tree of 32
+// lanes and one of the block per value: 16 meshes of 65,536 nodes in a batch 41.6 -> 39.2 ms, two
+// steps of 2,963,088 nodes 217.4 -> 211.9 ms.
+template <int NC>
+__device__ __forceinline__ bool seg_arrive(int item, int seg, const DSeg& G, const ItemList& IL,
+                                           const Red& red, double* res) {
+  constexpr int M = pow2_up(NC), NW = kBlock / 32;
+  __shared__ double sm[NW][M];
+  __shared__ int am_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(G.counter + seg, 1u);
+    am_last = (t == (unsigned)IL.seg_nitems[seg] - 1u);
+  }
+  __syncthreads();
+  if (!am_last) return false;
+  __threadfence();
+  const double* p = red.partial + (int64_t)IL.seg_item0[seg] * M;
+  const int ne = IL.seg_nitems[seg] * M;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  int e = threadIdx.x;
+  for (; e + 3 * kBlock < ne; e += 4 * kBlock) {
+    double x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = __ldcg(p + e + u * kBlock);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] += x[u];
+  }
+  for (; e < ne; e += kBlock) a[0] += __ldcg(p + e);
+  double acc = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+  for (int o = M; o < 32; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);
+  if (lane < M) sm[warp][lane] = acc;
+  __syncthreads();
+  if (threadIdx.x < NC) {
+    double x[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) x[w] = sm[w][threadIdx.x];
+#pragma unroll
+    for (int h = NW / 2; h >= 1; h >>= 1)
+#pragma unroll
+      for (int w = 0; w < h; ++w) x[w] += x[w + h];
+    res[threadIdx.x] = x[0];
+  }
+  if (threadIdx.x == 0) G.counter[seg] = 0u;
+  __syncthreads();
+  return true;
+}
+
+// Block reduction of NC values (v: padded with zeros to a power of two) into the item's partials,
+// then seg_arrive.  Blocks of kBlock threads.
+template <int NC, typename V>
+__device__ __forceinline__ bool seg_reduce_of(V (&v)[pow2_up(NC)], int item, int seg, const DSeg& G,
+                                              const ItemList& IL, const Red& red, double* res) {
+  constexpr int M = pow2_up(NC), NW = kBlock / 32, R = 32 / M;
+  __shared__ V sm[M][NW];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const V s = lane_sums<M, 32>(v);
+  if (lane % R == 0) sm[lane / R][warp] = s;
+  __syncthreads();
+  if (warp == 0) {
+    // NW lanes per value, 32 / NW values at a time
+#pragma unroll
+    for (int c0 = 0; c0 < NC; c0 += 32 / NW) {
+      const int c = c0 + lane / NW;
+      V x = sm[c < M ? c : 0][lane % NW];
+#pragma unroll
+      for (int o = NW / 2; o >= 1; o >>= 1) x = plus(x, lane_xor(x, o));
+      if (lane % NW == 0 && c < M) red.partial[(int64_t)item * M + c] = as_double(x);
+    }
+    __syncwarp();
+  }
+  return seg_arrive<NC>(item, seg, G, IL, red, res);
+}
+
+// the same for FP64 values
+template <int NC>
+__device__ __forceinline__ bool seg_reduce(double (&v)[NC], int item, int seg, const DSeg& G,
+                                           const ItemList& IL, const Red& red, double* res) {
+  double x[pow2_up(NC)];
+#pragma unroll
+  for (int c = 0; c < pow2_up(NC); ++c) x[c] = c < NC ? v[c < NC ? c : 0] : 0.0;
+  return seg_reduce_of<NC>(x, item, seg, G, IL, red, res);
 }
 
 // seg_reduce of per-thread values given as unevaluated sums hi + lo in T.  T = float: the warp
@@ -129,35 +200,11 @@ __device__ __forceinline__ bool seg_reduce_hl(const T (&hi)[NC], const T (&lo)[N
     for (int c = 0; c < NC; ++c) v[c] = hi[c] + lo[c];
     return seg_reduce<NC>(v, item, seg, G, IL, red, res);
   } else {
-    __shared__ float smh[NC][32], sml[NC][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    DF x[pow2_up(NC)];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      float h = hi[c], l = lo[c];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float bh = __shfl_down_sync(kFull, h, o), bl = __shfl_down_sync(kFull, l, o);
-        df_add(h, l, bh, bl);
-      }
-      if (lane == 0) {
-        smh[c][warp] = h;
-        sml[c][warp] = l;
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        float h = lane < nw ? smh[c][lane] : 0.f, l = lane < nw ? sml[c][lane] : 0.f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float bh = __shfl_down_sync(kFull, h, o), bl = __shfl_down_sync(kFull, l, o);
-          df_add(h, l, bh, bl);
-        }
-        if (lane == 0) red.partial[(int64_t)item * kRedComp + c] = (double)h + (double)l;
-      }
-    }
-    return seg_arrive<NC>(item, seg, G, IL, red, res);
+    for (int c = 0; c < pow2_up(NC); ++c)
+      x[c] = c < NC ? DF{hi[c < NC ? c : 0], lo[c < NC ? c : 0]} : DF{0.f, 0.f};
+    return seg_reduce_of<NC>(x, item, seg, G, IL, red, res);
   }
 }
 
