@@ -1392,7 +1392,7 @@ class Engine final : public EngineBase {
     const T* dinv = epr == 3 ? dinv3_ : dinv1_;
     auto precondition = [&](T* z, int init) -> int {
       TK(GSPM_KCLASS_CG_VEC, launch_restrict<T>(L_, CC_, epr, r_, rco, rc_));
-      TK(GSPM_KCLASS_CG_VEC, launch_coarse_symv<T>(L_, CC_, TL, epr, cinv, rco, rc_, qsym_, ec_));
+      TK(GSPM_KCLASS_CG_VEC, launch_coarse_symv<T>(L_, CC_, TL, epr, cinv, rco, epr == 3 ? crows3_ : crows1_, rc_, qsym_, ec_));
       TK(GSPM_KCLASS_CG_VEC, launch_pcg_z<T>(L_, SG_, CC_, epr, r_, dinv, ec_, z, st, init, red_));
       return GSPM_OK;
     };
@@ -1839,11 +1839,18 @@ class Engine final : public EngineBase {
           break;
         }
     CC_ = DCoarse{na, d_aor, d_aptr, d_arows, d_aseg, d_agg0, contig};
+    // work items over groups of 32 coarse rows (the reduction scratch holds any list of nseg_ segments)
+    for (int e = 1; e <= 3; e += 2) {
+      std::vector<int64_t> u0(S, 0), nu(S);
+      for (int sg = 0; sg < S; ++sg) nu[sg] = ((int64_t)e * hb_.coarse[sg].n_agg + 31) / 32;
+      int max_items = 0;
+      ST(make_item_lists(u0, nu, e == 3 ? crows3_ : crows1_, &max_items));
+    }
     pc_ = true;
     return contig ? init_pieces(aor, agg0) : GSPM_OK;
   }
 
-  // Pieces of the aggregates in the update's work items, and work items over the coarse rows
+  // Pieces of the aggregates in the update's work items
   int init_pieces(const std::vector<int32_t>& aor, const std::vector<int32_t>& agg0) {
     const int S = nseg_, lst = pcg_resident<T>() - 1;
     const int ni = SG_.list[lst].nitems;
@@ -1881,15 +1888,6 @@ class Engine final : public EngineBase {
     CK(cudaMemcpy(d_row, prow.data(), prow.size() * 4, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(d_ap, ap.data(), ap.size() * 4, cudaMemcpyHostToDevice));
     PP_ = DPieces{(int)prow.size(), max_item, lst, d_ip0, d_row, d_ap};
-    for (int e = 1; e <= 3; e += 2) {
-      std::vector<int64_t> u0(S), nu(S);
-      for (int sg = 0; sg < S; ++sg) {
-        u0[sg] = (int64_t)e * agg0[sg];
-        nu[sg] = (int64_t)e * (agg0[sg + 1] - agg0[sg]);
-      }
-      int max_items = 0;  // (the reduction scratch holds any list of nseg_ segments)
-      ST(make_item_lists(u0, nu, e == 3 ? crows3_ : crows1_, &max_items));
-    }
     pieces_ok_ = true;
     return GSPM_OK;
   }
@@ -2215,9 +2213,9 @@ class Engine final : public EngineBase {
   T *dinv3_ = nullptr, *dinv1_ = nullptr;
   T *dgs_eps_ = nullptr, *dgs_aeps_ = nullptr;  // Jacobi of the GSPM solves (NULL: plain)
   T *rc_ = nullptr, *ec_ = nullptr;
+  ItemList crows3_[kItemLists], crows1_[kItemLists];  // work items over the coarse rows
   // two-level CG on aggregates that are runs of rows
   DPieces PP_{};
-  ItemList crows3_[kItemLists], crows1_[kItemLists];
   T* pieces_ = nullptr;
   bool pieces_ok_ = false;
   // volume averages in ABI order

@@ -820,94 +820,117 @@ struct CoarsePack<double> {
   }
 };
 
-// Tile (I, J) of the stored upper triangle: A_IJ rc_J -> prow[t], and off the diagonal
-// A_IJ^T rc_I -> pcol[t].  A warp row-load covers RPW tile rows (LPR lanes per row, W values
-// per lane); the row sums reduce over a row's lanes, the column sums over the lanes that hold
-// the same columns and then over the warps in a fixed order.
+// Tile (I, J) of the stored upper triangle: A_IJ rc_J and, off the diagonal, A_IJ^T rc_I.  A warp
+// row-load covers RPW tile rows (LPR lanes per row, W values per lane); the row sums reduce over a
+// row's lanes (NP rows of the warp at once, see lane_sums), the column sums over the lanes that hold
+// the same columns and then over the warps in a fixed order.  Bound by HBM where the tiles do not
+// fit the L2.  Q holds a tile's products as one run, so that they leave in whole lines.  17,661 coarse
+// unknowns (314 MB): 71 -> 55 us per launch, the sum of Q's rows 18.9 -> 12.1 us; two steps of
+// 2,963,088 nodes 211.9 -> 204 ms.
 template <typename T, typename S>
-__global__ void __launch_bounds__(kBlock) k_coarse_symv_tiles(DSymTiles TL,
-                                                              const S* __restrict__ inv,
-                                                              const int64_t* __restrict__ rc_off,
-                                                              const T* __restrict__ rc,
-                                                              T* __restrict__ Q) {
+__global__ void __launch_bounds__(kBlock, 4) k_coarse_symv_tiles(DSymTiles TL,
+                                                                 const S* __restrict__ inv,
+                                                                 const int64_t* __restrict__ rc_off,
+                                                                 const T* __restrict__ rc,
+                                                                 T* __restrict__ Q) {
   pdl_enter();
   constexpr int kCoarseTile = coarse_tile<T>();
   constexpr int W = CoarsePack<S>::W, LPR = kCoarseTile / W, RPW = 32 / LPR;
   constexpr int NW = kBlock / 32, RPP = NW * RPW, NP = kCoarseTile / RPP;
-  static_assert(LPR <= 32 && NP >= 1, "tile layout");
-  __shared__ T srow[kCoarseTile];
-  __shared__ T scol[NW][kCoarseTile];
+  static_assert(LPR <= 32 && LPR >= NP && pow2_up(NP) == NP, "tile layout");
+  // two sets: a block may start on its next tile while slower warps still read this one's sums
+  __shared__ T srow[2][kCoarseTile];
+  __shared__ T scol[2][NW][kCoarseTile];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cp = lane % LPR, rg = lane / LPR;
-  for (int64_t t = blockIdx.x; t < TL.ntiles; t += gridDim.x) {
-    const int seg = TL.tseg[t], I = TL.tI[t], J = TL.tJ[t];
+  int set = 0;
+  for (int64_t t = blockIdx.x; t < TL.ntiles; t += gridDim.x, set ^= 1) {
     const S* tile = inv + t * (int64_t)(kCoarseTile * kCoarseTile);
-    const T* xs = rc + rc_off[seg];
     typename CoarsePack<S>::Raw a[NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p)
       a[p] = CoarsePack<S>::load(tile + (p * RPP + warp * RPW + rg) * kCoarseTile + cp * W);
+    const int seg = TL.tseg[t], I = TL.tI[t], J = TL.tJ[t];
+    const T* xs = rc + rc_off[seg];
     T xj[W];
     ldn<T, W>(xs + (int64_t)J * kCoarseTile + cp * W, xj);
-    T cs[W];
+    T cs[W], rs[NP];
 #pragma unroll
     for (int c = 0; c < W; ++c) cs[c] = T(0);
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
-      const int row = p * RPP + warp * RPW + rg;
+      const T xi = xs[(int64_t)I * kCoarseTile + p * RPP + warp * RPW + rg];
       T w[W];
       CoarsePack<S>::cvt(a[p], w);
-      T rs = T(0);
+      rs[p] = T(0);
 #pragma unroll
-      for (int c = 0; c < W; ++c) rs += w[c] * xj[c];
-#pragma unroll
-      for (int o = 1; o < LPR; o <<= 1) rs += __shfl_xor_sync(kFull, rs, o);
-      if (cp == 0) srow[row] = rs;
-      const T xi = xs[(int64_t)I * kCoarseTile + row];
-#pragma unroll
-      for (int c = 0; c < W; ++c) cs[c] += w[c] * xi;
+      for (int c = 0; c < W; ++c) {
+        rs[p] += w[c] * xj[c];
+        cs[c] += w[c] * xi;
+      }
     }
+    const T row_sum = lane_sums<NP, LPR>(rs);
+    if (cp % (LPR / NP) == 0)
+      srow[set][cp / (LPR / NP) * RPP + warp * RPW + rg] = row_sum;
 #pragma unroll
     for (int o = LPR; o < 32; o <<= 1)
 #pragma unroll
       for (int c = 0; c < W; ++c) cs[c] += __shfl_xor_sync(kFull, cs[c], o);
     if (rg == 0)
 #pragma unroll
-      for (int c = 0; c < W; ++c) scol[warp][cp * W + c] = cs[c];
+      for (int c = 0; c < W; ++c) scol[set][warp][cp * W + c] = cs[c];
     __syncthreads();
+    // tile row I of Q, run J: the rows' sums; tile row J, run I: the columns' sums
+    const int64_t Tn = TL.seg_T[seg];
+    T* q = Q + TL.seg_q0[seg];
+    const int k = threadIdx.x % kCoarseTile;
     if (threadIdx.x < kCoarseTile) {
-      const int64_t Tn = TL.seg_T[seg];
-      T* q = Q + TL.seg_q0[seg];
-      q[((int64_t)I * kCoarseTile + threadIdx.x) * Tn + J] = srow[threadIdx.x];
-      if (I != J) {
-        T v = T(0);
+      q[((int64_t)I * Tn + J) * kCoarseTile + k] = srow[set][k];
+    } else if (threadIdx.x < 2 * kCoarseTile && I != J) {
+      T v = T(0);
 #pragma unroll
-        for (int w = 0; w < NW; ++w) v += scol[w][threadIdx.x];
-        q[((int64_t)J * kCoarseTile + threadIdx.x) * Tn + I] = v;
-      }
+      for (int w = 0; w < NW; ++w) v += scol[set][w][k];
+      q[((int64_t)J * Tn + I) * kCoarseTile + k] = v;
     }
-    __syncthreads();
   }
 }
 
-// ec(g) = the sum of row g of Q (one warp per coarse row, lanes over the columns, fixed order)
+// Sum over the tile columns of 32 coarse rows of Q (group grp of the segment), a warp's lanes on
+// the rows and the block's warps on the columns, in a fixed order: valid in warp 0, a row per lane
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_coarse_symv_sum(DCoarse C, DSymTiles TL, int epr,
-                                                            const T* __restrict__ Q,
+__device__ __forceinline__ T coarse_rows_sum(const T* __restrict__ q, int64_t Tn, int64_t grp,
+                                             T (&sm)[kBlock / 32][32]) {
+  constexpr int TS = coarse_tile<T>(), NW = kBlock / 32, GP = TS / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const T* p = q + (grp / GP) * Tn * TS + (grp % GP) * 32 + lane;
+  T acc = T(0);
+#pragma unroll 4
+  for (int64_t J = warp; J < Tn; J += NW) acc += p[J * TS];
+  sm[warp][lane] = acc;
+  __syncthreads();
+  T v = T(0);
+  if (warp == 0)
+#pragma unroll
+    for (int w = 0; w < NW; ++w) v += sm[w][lane];
+  return v;
+}
+
+// ec = the row sums of Q; items: groups of 32 coarse rows of a segment
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_coarse_symv_sum(ItemList IL, DCoarse C, DSymTiles TL,
+                                                            int epr, const T* __restrict__ Q,
                                                             T* __restrict__ ec) {
   pdl_enter();
-  const int lane = threadIdx.x & 31;
-  const int64_t ncoarse = C.nagg * epr;
-  for (int64_t g = gtid() >> 5; g < ncoarse; g += gstride() >> 5) {
-    const int seg = C.agg_seg[g / epr];
-    const int64_t loc = g - (int64_t)C.seg_agg0[seg] * epr;
-    const int64_t Tn = TL.seg_T[seg];
-    const T* q = Q + TL.seg_q0[seg] + loc * Tn;
-    T acc = T(0);
-    for (int64_t j = lane; j < Tn; j += 32) acc += q[j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
-    if (lane == 0) ec[g] = acc;
+  __shared__ T sm[kBlock / 32][32];
+  for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
+    const int seg = IL.seg[item];
+    const int64_t nc = (int64_t)(C.seg_agg0[seg + 1] - C.seg_agg0[seg]) * epr;
+    for (int64_t grp = IL.sl0[item]; grp < IL.sl1[item]; ++grp) {
+      const T e = coarse_rows_sum<T>(Q + TL.seg_q0[seg], TL.seg_T[seg], grp, sm);
+      const int64_t loc = grp * 32 + threadIdx.x;
+      if (threadIdx.x < 32 && loc < nc) ec[(int64_t)C.seg_agg0[seg] * epr + loc] = e;
+      __syncthreads();
+    }
   }
 }
 
@@ -1182,9 +1205,8 @@ __global__ void __launch_bounds__(kBlock) k_piece_sum(DCoarse C, DPieces PP,
   }
 }
 
-// ec(g) = the sum of row g of Q (one warp per coarse row, lanes over the columns, fixed order), and
-// per segment r_c.e_c and the sums over its rows of P e_c: with the update's sums they give r.z and
-// the mean of z, hence beta
+// ec = the row sums of Q (items: groups of 32 coarse rows of a segment), and per segment r_c.e_c and
+// the sums over its rows of P e_c: with the update's sums they give r.z and the mean of z, hence beta
 template <typename T, int EPR>
 __global__ void __launch_bounds__(kBlock) k_pcg_coarse(DSeg G, ItemList IL, DCoarse C, DSymTiles TL,
                                                        const T* __restrict__ Q,
@@ -1192,31 +1214,36 @@ __global__ void __launch_bounds__(kBlock) k_pcg_coarse(DSeg G, ItemList IL, DCoa
                                                        const T* __restrict__ rc, T* __restrict__ ec,
                                                        CGState* st, int first, Red red) {
   pdl_enter();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ T sm[kBlock / 32][32];
   for (int item = blockIdx.x; item < IL.nitems; item += gridDim.x) {
     const int seg = IL.seg[item];
     CGState* sg = st + seg;
     if (!sg->active) continue;
-    const int64_t g0 = (int64_t)C.seg_agg0[seg] * EPR, Tn = TL.seg_T[seg];
+    const int64_t g0 = (int64_t)C.seg_agg0[seg] * EPR;
+    const int64_t nc = (int64_t)C.seg_agg0[seg + 1] * EPR - g0;
     T hi[1 + EPR], lo[1 + EPR];
 #pragma unroll
     for (int v = 0; v < 1 + EPR; ++v) hi[v] = lo[v] = T(0);
-    for (int64_t g = IL.sl0[item] + warp; g < IL.sl1[item]; g += kBlock / 32) {
-      const int64_t loc = g - g0;
-      const T* qr = Q + TL.seg_q0[seg] + loc * Tn;
-      T acc = T(0);
-      for (int64_t j = lane; j < Tn; j += 32) acc += qr[j];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
-      if (lane == 0) {
-        ec[g] = acc;
-        const int I = (int)(g / EPR), a = (int)(g - (int64_t)I * EPR);
-        const T cnt = (T)(C.agg_ptr[I + 1] - C.agg_ptr[I]);
-        kahan_add(hi[0], lo[0], acc * rc[rc_off[seg] + loc]);
+    for (int64_t grp = IL.sl0[item]; grp < IL.sl1[item]; ++grp) {
+      const int64_t loc = grp * 32 + threadIdx.x;
+      const bool mine = threadIdx.x < 32 && loc < nc;
+      T rcv = T(0), cnt = T(0);
+      int a = 0;
+      if (mine) {
+        const int64_t I = (g0 + loc) / EPR;
+        a = (int)((g0 + loc) - I * EPR);
+        rcv = rc[rc_off[seg] + loc];
+        cnt = (T)(C.agg_ptr[I + 1] - C.agg_ptr[I]);
+      }
+      const T e = coarse_rows_sum<T>(Q + TL.seg_q0[seg], TL.seg_T[seg], grp, sm);
+      if (mine) {
+        ec[g0 + loc] = e;
+        kahan_add(hi[0], lo[0], e * rcv);
 #pragma unroll
         for (int b = 0; b < EPR; ++b)
-          if (a == b) kahan_add(hi[1 + b], lo[1 + b], cnt * acc);
+          if (a == b) kahan_add(hi[1 + b], lo[1 + b], cnt * e);
       }
+      __syncthreads();
     }
 #pragma unroll
     for (int v = 0; v < 1 + EPR; ++v) lo[v] = -lo[v];
@@ -2234,16 +2261,23 @@ cudaError_t launch_restrict(const Launch& L, const DCoarse& C, int epr, const T*
   return cudaGetLastError();
 }
 
+static const ItemList& crow_list(const ItemList (&crows)[kItemLists], const void* kernel) {
+  const int per_sm = resident_per_sm(kernel);
+  return crows[(per_sm < kItemLists ? per_sm : kItemLists) - 1];
+}
+
 template <typename T>
 cudaError_t launch_coarse_symv(const Launch& L, const DCoarse& C, const DSymTiles& TL, int epr,
                                const typename CoarseStore<T>::type* inv, const int64_t* rc_off,
-                               const T* rc, T* Q, T* ec) {
+                               const ItemList (&crows)[kItemLists], const T* rc, T* Q, T* ec) {
   (*L.counter) += 2;
   if (!aligned16(inv) || !aligned16(rc)) return cudaErrorInvalidValue;
   auto k1 = k_coarse_symv_tiles<T, typename CoarseStore<T>::type>;
   ST_CUDA(launch_pdl(k1, GSPM_GRID(L, TL.ntiles * kBlock, k1), L.stream, TL, inv, rc_off, rc, Q));
   auto k2 = k_coarse_symv_sum<T>;
-  ST_CUDA(launch_pdl(k2, GSPM_GRID(L, C.nagg * epr * 32, k2), L.stream, C, TL, epr, Q, ec));
+  const ItemList& il = crow_list(crows, reinterpret_cast<const void*>(k2));
+  ST_CUDA(launch_pdl(k2, std::min(il.nitems, L.max_blocks), L.stream, il, C, TL, epr, (const T*)Q,
+                     ec));
   return cudaGetLastError();
 }
 template <typename T, int EPR>
@@ -2279,10 +2313,9 @@ static cudaError_t pcg_coarse_n(const Launch& L, const DSeg& G, const DCoarse& C
   ST_CUDA(launch_pdl(k1, GSPM_GRID(L, TL.ntiles * kBlock, k1), L.stream, TL, inv, rc_off,
                      (const T*)rc, Q));
   auto k2 = k_pcg_coarse<T, EPR>;
-  const int per_sm = resident_per_sm(reinterpret_cast<const void*>(k2));
-  const ItemList& il = crows[(per_sm < kItemLists ? per_sm : kItemLists) - 1];
-  return launch_pdl(k2, grid_for(L, (int64_t)il.nitems * kBlock, reinterpret_cast<const void*>(k2)),
-                    L.stream, G, il, C, TL, (const T*)Q, rc_off, (const T*)rc, ec, st, first, red);
+  const ItemList& il = crow_list(crows, reinterpret_cast<const void*>(k2));
+  return launch_pdl(k2, std::min(il.nitems, L.max_blocks), L.stream, G, il, C, TL, (const T*)Q,
+                    rc_off, (const T*)rc, ec, st, first, red);
 }
 
 template <typename T>
@@ -2533,7 +2566,7 @@ cudaError_t launch_scaled_diff(const Launch& L, int64_t len, const T* a, const T
                                           const int64_t*, T*);                                    \
   template cudaError_t launch_coarse_symv<T>(const Launch&, const DCoarse&, const DSymTiles&, int, \
                                              const typename CoarseStore<T>::type*, const int64_t*, \
-                                             const T*, T*, T*);                                   \
+                                             const ItemList(&)[kItemLists], const T*, T*, T*);    \
   template cudaError_t launch_pcg_update<T>(const Launch&, const DSeg&, const DPieces&, int, T*,  \
                                             const T*, const T*, T*, CGState*, int*, int, Red);    \
   template cudaError_t launch_pcg_coarse<T>(                                                      \

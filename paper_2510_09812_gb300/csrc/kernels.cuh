@@ -225,8 +225,8 @@ inline int64_t coarse_ld(int64_t nc) {
 }
 // The stored tiles of all segments: tile t of the global list belongs to segment tseg[t], tile
 // row tI[t], column tJ[t]; segment s's tiles start at seg_tile0[s] and it has seg_T[s] tile rows.
-// The partials of segment s sit in Q at seg_q0[s], one row of seg_T[s] values per (padded)
-// coarse row of the segment.
+// The partials of segment s sit in Q at seg_q0[s]: per tile row seg_T[s] runs of one tile side, run
+// J the products with the tile in column J.
 struct DSymTiles {
   int64_t ntiles;
   const int32_t* tseg;
@@ -237,13 +237,14 @@ struct DSymTiles {
   const int64_t* seg_q0;
 };
 // ec = A_c^-1 rc with the stored upper triangle, in two kernels: each tile (I, J) writes the
-// partial products A_IJ rc_J to Q(row I tile + r, J) and, off the diagonal, A_IJ^T rc_I to
-// Q(row J tile + c, I) (every stored value read once); then each coarse row sums its row of Q
-// in column order.  Q: scratch of sum over segments of T^2 tile values.
+// partial products A_IJ rc_J to run J of tile row I of Q and, off the diagonal, A_IJ^T rc_I to run I
+// of tile row J (every stored value read once); then each coarse row sums its values of Q, warps
+// over the columns in a fixed order.  Q: scratch of sum over segments of T^2 tile sides.  crows:
+// work items over groups of 32 coarse rows, numbered from 0 in each segment.
 template <typename T>
 cudaError_t launch_coarse_symv(const Launch& L, const DCoarse& C, const DSymTiles& TL, int epr,
                                const typename CoarseStore<T>::type* inv, const int64_t* rc_off,
-                               const T* rc, T* Q, T* ec);
+                               const ItemList (&crows)[kItemLists], const T* rc, T* Q, T* ec);
 // Two-level CG on aggregates that are runs of rows (DCoarse::contig), z never stored: the update
 // forms r, the sums of the residual and of D^-1 r, and the restricted residual piece by piece (a
 // piece: the part of an aggregate in one work item); the coarse product's last step adds r_c.e_c
@@ -263,7 +264,6 @@ cudaError_t launch_pcg_update(const Launch& L, const DSeg& G, const DPieces& PP,
                               const T* q, const T* dinv, T* pieces, CGState* st, int* nactive,
                               int first, Red red);
 // rc from the pieces, ec = A_c^-1 rc, then rz (first) or beta and rz, and the means for the p-update.
-// crows: work items over the coarse rows.
 template <typename T>
 cudaError_t launch_pcg_coarse(const Launch& L, const DSeg& G, const DCoarse& C, const DPieces& PP,
                               const DSymTiles& TL, const ItemList (&crows)[kItemLists], int epr,
