@@ -1034,9 +1034,12 @@ __global__ void __launch_bounds__(kBlock) k_pcg_z(DSeg G, ItemList IL, DCoarse C
 // takes x along because it reads p anyway.  A step of 2,963,088 nodes (two of 548 two-level
 // iterations): 217.3 -> 213.5 ms; 16 meshes of 65,536 nodes: 43.2 -> 41.6 ms.
 //
-// Four rows per thread and round (whole 16-byte packs: item ranges start at multiples of 32 rows).
-// A warp's 128 rows lie in one or two aggregates: it sums each by shuffles into its own slot of the
-// piece, and the block's eight slots are added at the end (no barrier per aggregate).
+// Four rows per thread and round (whole 16-byte packs: item ranges start at multiples of 32 rows),
+// a warp on a run of 128-row groups.  A lane adds up its rows of the current piece and the warp sums
+// over its lanes only where a piece ends (a few per warp), into its own slot of the piece; the
+// block's eight slots are added at the end (no barrier per aggregate).  Summing the lanes for every
+// group of rows took 32.5 us per launch at 2,963,088 nodes (three components), this takes 30.2; the
+// restriction in a kernel of its own and the update 15.9 + 33.6.
 template <typename T, int EPR>
 __global__ void __launch_bounds__(kBlock, pcg_resident<T>())
     k_pcg_update(DSeg G, ItemList IL, DPieces PP, T* __restrict__ r, const T* __restrict__ q,
@@ -1065,8 +1068,27 @@ __global__ void __launch_bounds__(kBlock, pcg_resident<T>())
     T rr = T(0), dz = T(0), dzc = T(0), sr[EPR], sd[EPR];
 #pragma unroll
     for (int a = 0; a < EPR; ++a) sr[a] = sd[a] = T(0);
-    int pc = 0;
-    for (int64_t w0 = r0 + 128 * warp; w0 < r1; w0 += 128 * NW) {
+    const int64_t run = ((r1 - r0 + 127) / 128 + NW - 1) / NW * 128;
+    const int64_t wb = r0 + run * warp, we = wb + run < r1 ? wb + run : r1;
+    // the piece that holds the warp's first row
+    int pc = -1;
+    for (int k = 0; k < np; k += 32)
+      pc += __popc(__ballot_sync(kFull, k + lane < np && PP.row[p0 + k + lane] <= wb));
+    int64_t pend = pc + 1 < np ? (int64_t)PP.row[p0 + pc + 1] : r1;  // its end
+    T acc[EPR];
+#pragma unroll
+    for (int a = 0; a < EPR; ++a) acc[a] = T(0);
+    auto close_piece = [&]() {
+#pragma unroll
+      for (int a = 0; a < EPR; ++a) {
+        T v = acc[a];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
+        if (lane == 0) ps[(pc * NW + warp) * EPR + a] = v;
+        acc[a] = T(0);
+      }
+    };
+    for (int64_t w0 = wb; w0 < we; w0 += 128) {
       const int64_t row = w0 + 4 * lane;
       T rv[N];
 #pragma unroll
@@ -1113,28 +1135,27 @@ __global__ void __launch_bounds__(kBlock, pcg_resident<T>())
             }
           }
       }
-      // pieces of the warp's rows
-      while (pc + 1 < np && PP.row[p0 + pc + 1] <= w0) ++pc;
-      for (int k = pc; k < np; ++k) {
-        const int64_t b = PP.row[p0 + k];
-        if (b >= w0 + 128) break;
-        const int64_t e = k + 1 < np ? (int64_t)PP.row[p0 + k + 1] : r1;
-        T v[EPR];
-#pragma unroll
-        for (int a = 0; a < EPR; ++a) v[a] = T(0);
+      // the pieces that end within the warp's 128 rows, then the rows of the one that goes on (rows
+      // past the item hold zeros)
+      int64_t from = w0;
+      while (pend < w0 + 128 && pend < r1) {
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          if (row + u >= b && row + u < e)
+          if (row + u >= from && row + u < pend)
 #pragma unroll
-            for (int a = 0; a < EPR; ++a) v[a] += rv[u * EPR + a];
-#pragma unroll
-        for (int a = 0; a < EPR; ++a) {
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) v[a] += __shfl_down_sync(kFull, v[a], o);
-          if (lane == 0) ps[(k * NW + warp) * EPR + a] += v[a];
-        }
+            for (int a = 0; a < EPR; ++a) acc[a] += rv[u * EPR + a];
+        close_piece();
+        from = pend;
+        ++pc;
+        pend = pc + 1 < np ? (int64_t)PP.row[p0 + pc + 1] : r1;
       }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (row + u >= from)
+#pragma unroll
+          for (int a = 0; a < EPR; ++a) acc[a] += rv[u * EPR + a];
     }
+    if (wb < we) close_piece();
     __syncthreads();
     for (int k = threadIdx.x; k < np * EPR; k += kBlock) {
       T v = T(0);
