@@ -1211,12 +1211,15 @@ class Engine final : public EngineBase {
 
   // shared memory of a fused loop (227 KB per block less its static part)
   static constexpr size_t kLoopSmem = 232448 - 4096;
-  // Rows up to which the fused loops run: one mesh, and a batch (whose meshes share the blocks less
-  // evenly and do not converge together).  Mixed precision, ms per step, fused against separate
-  // kernels: 198,400 nodes 12.4 / 22.3, 300,000 15.0 / 23.2, 396,000 20.1 / 26.0, 524,288 25.6 / 29.8;
-  // batches of 252,432 nodes 14.6 / 23.1, 347,296 (FP64) 57.4 / 84.1, 513,808 29.4 / 27.3, 1,138,576
-  // 67.2 / 43.6.
-  static constexpr int64_t kLoopRows = 600000, kLoopBatchRows = 400000;
+  // Rows up to which the fused loops run: one mesh, and a batch (whose meshes are groups of blocks
+  // that wait only among themselves and stop one by one).  Beyond, a block's vectors outgrow its
+  // shared memory and the packets of p, twice the bytes, the L2's share.  ms, fused / separate
+  // kernels: two mixed steps at 66,816 nodes 13.3 / 25.1, 198,400 24.0 / 34.2, 300,000 29.1 / 35.2,
+  // 396,000 39.5 / 42.0, 449,280 55.9 / 44.6, 524,288 50.2 / 48.8; FP64 100,800 45.9 / 58.9, 198,400
+  // 77.4 / 84.8, 300,000 103.4 / 104.0, 396,000 147.7 / 132.8; elastic solves 152,969 6.9 / 9.3,
+  // 300,000 11.5 / 12.2, 396,000 16.0 / 14.4, FP64 300,000 33.6 / 30.6; batches 82,064 7.3 / 12.0,
+  // 252,432 14.1 / 17.6, 347,296 16.3 / 20.6, FP64 347,296 56.8 / 68.0, 513,808 29.4 / 27.3.
+  static constexpr int64_t kLoopRows = sizeof(T) == 4 ? 400000 : 280000, kLoopBatchRows = 400000;
 
   template <typename X>
   int upload(T** dst, const std::vector<X>& src) {

@@ -27,8 +27,8 @@
 // together.
 //
 // Measured (separate kernels -> fused): time steps at 1,024 nodes (FP64) 7.8 -> 3.1 ms, 19,305 nodes
-// (mixed) 14.8 -> 5.8, 65,536 (mixed) 18.4 -> 7.0, 65,536 hexahedra (FP64) 22.6 -> 12.6, 524,288
-// (mixed) 30.8 -> 26.4; an elastic solve at 152,969 nodes 13.9 -> 7.4 ms.  An iteration of K^mech at
+// (mixed) 14.8 -> 5.8, 65,536 (mixed) 18.4 -> 7.0, 65,536 hexahedra (FP64) 22.6 -> 12.6; an elastic
+// solve at 152,969 nodes 13.9 -> 7.4 ms; larger sizes at kLoopRows.  An iteration of K^mech at
 // 19,305 nodes takes 43,000 cycles: 5,000 for the product, 2,500 for the vectors, the rest the chain
 // of exchanges (two hops for p.q, three for the residual and the coarse correction, one for p).  What
 // bounds it is that chain of dependent hops and single-warp sums, not bandwidth; at 65,536 hexahedra

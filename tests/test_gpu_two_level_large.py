@@ -1,6 +1,6 @@
 """Two-level CG in separate kernels with z never stored (aggregates that are runs of rows).
 
-It runs where the fused loops do not: above 600,000 nodes, and in batches of more meshes than the GPU
+It runs where the fused loops do not: above 400,000 nodes (mixed precision), and in batches of more meshes than the GPU
 has SMs.  References: the same systems with ordering "none" (aggregates that are not runs of rows,
 z stored) and each mesh of a batch alone.  FP64 solves to 1e-12 agree within the CG error (1e-9 of
 a field's largest value), mixed steps at 1e-7 within the mixed-precision bound of 1e-4 rad; replayed
