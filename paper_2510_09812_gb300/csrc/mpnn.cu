@@ -677,15 +677,35 @@ __global__ void __launch_bounds__(kThreads) k_in_bwd(int64_t n, const float* __r
   if (t < kHid) pp[kFeat * kHid + t] = db;
 }
 
-// grad[k] = sum over blocks of part[b][k], k < count; part[b][count] to *last where there is one.
+// The block partials of one gradient: out[k] = sum over blocks b < nblocks of part[b][k], k < count,
+// and part[b][count] to *last where there is one.  first: its first block of k_reduce_parts.
+struct Parts {
+  int nblocks, count, stride, first;
+  const float* part;
+  float *out, *last;
+};
+constexpr int kPartSets = kLayers + 2;  // W_out (with the loss), the layers, W_in
+struct PartList {
+  Parts p[kPartSets];
+};
+
 // A block sums 32 values: eight groups of threads take every eighth partial, eight loads in flight,
 // then the groups in order (13 us for 304 partials of 8,256 values; one thread per value 57 us).
-__global__ void __launch_bounds__(kThreads) k_reduce_parts(int nblocks, int count, int stride,
-                                                           const float* __restrict__ part,
-                                                           float* __restrict__ grad,
-                                                           float* __restrict__ last) {
+// All gradients in one launch: bound by the latency of its longest sum (1,024 partials of W_out's
+// 196 values, 12 us), which alone or beside the layers' takes the same time; a launch per gradient
+// took 41 us of device time.  Loss and gradients at 65,536 nodes: 513 -> 495 us.
+__global__ void __launch_bounds__(kThreads) k_reduce_parts(PartList PL) {
   __shared__ float sm[8][32];
-  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
+  int set = 0;
+#pragma unroll
+  for (int i = 1; i < kPartSets; ++i)
+    if ((int)blockIdx.x >= PL.p[i].first) set = i;
+  const Parts& P = PL.p[set];
+  const int nblocks = P.nblocks, count = P.count, stride = P.stride;
+  const float* __restrict__ part = P.part;
+  float *grad = P.out, *last = P.last;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int k = ((int)blockIdx.x - P.first) * 32 + lane;
   const bool ok = k < count + (last ? 1 : 0);
   float s = 0.f;
   for (int b = g; ok && b < nblocks; b += 64) {
@@ -747,14 +767,6 @@ static inline int grid_bwd(const Launch& L, int64_t n) {
   const int64_t b = (n + kBwdRows - 1) / kBwdRows, cap = 2 * (int64_t)L.sms;
   return (int)(b > cap ? cap : b);
 }
-static cudaError_t reduce_parts(const Launch& L, int nblocks, int count, int stride,
-                                const float* part, float* grad, float* last) {
-  (*L.counter) += 1;
-  k_reduce_parts<<<(count + (last ? 1 : 0) + 31) / 32, kThreads, 0, L.stream>>>(
-      nblocks, count, stride, part, grad, last);
-  return cudaGetLastError();
-}
-
 template <typename T>
 cudaError_t mpnn_features(const Launch& L, int64_t n, const T* m, int64_t ld, const uint8_t* mag,
                           const T* up, const T* up2, double l100, double l111,
@@ -814,30 +826,44 @@ cudaError_t mpnn_backward(const Launch& L, int64_t n, const DSell& S, const Mpnn
   // grad layout = parameter layout: W_in, b_in, {W_l, b_l} x 3, W_out, b_out
   const int gb = grid_rows(L, n), gt = grid_bwd(L, n);
   cudaError_t e;
-  const int wout = kHid * 3 + 4;
+  // every gradient's block partials stay until the one reduction at the end: gb rows of W_out, b_out
+  // and the loss, then gt rows per layer and of W_in, less than max_blocks rows of a layer in all
+  // (gb <= max_blocks = 8 SMs, gt <= 2 SMs)
+  const int wout = kHid * 3 + 4, wl = 2 * kHid * kHid + kHid, wi = kFeat * kHid + kHid;
+  static_assert(8 * (kHid * 3 + 4) + 2 * kLayers * (2 * kHid * kHid + kHid) +
+                        2 * (kFeat * kHid + kHid) <= 8 * (2 * kHid * kHid + kHid),
+                "partials exceed the scratch");
+  PartList PL;
+  int set = 0, blocks = 0;
+  float* pp = part;
+  auto add = [&](int nblocks, int count, int stride, float* out, float* last) {
+    PL.p[set++] = Parts{nblocks, count, stride, blocks, pp, out, last};
+    blocks += (count + (last ? 1 : 0) + 31) / 32;
+    float* at = pp;
+    pp += (int64_t)nblocks * stride;
+    return at;
+  };
   (*L.counter) += 1;
-  k_out_bwd<<<gb, kThreads, 0, L.stream>>>(n, Y, T, H[kLayers], W.Wout, dHa, part);
-  // W_out, b_out, and the loss
-  if ((e = reduce_parts(L, gb, wout - 1, wout, part, grad + kOffWout, loss)) != cudaSuccess) return e;
+  k_out_bwd<<<gb, kThreads, 0, L.stream>>>(n, Y, T, H[kLayers], W.Wout, dHa,
+                                           add(gb, wout - 1, wout, grad + kOffWout, loss));
   float* dH = dHa;
   float* dHp = dHb;
-  const int wl = 2 * kHid * kHid + kHid;
   const size_t sm = mpnn_layer_bwd_smem();
   for (int l = kLayers - 1; l >= 0; --l) {
     (*L.counter) += 2;
     k_layer_bwd<<<gt, kThreads, sm, L.stream>>>(n, dH, H[l + 1], H[l], Z[l], W.Wf[l], dHp, dZ,
-                                                part);
-    if ((e = reduce_parts(L, gt, wl, wl, part, grad + kOffW[l], nullptr)) != cudaSuccess) return e;
+                                                add(gt, wl, wl, grad + kOffW[l], nullptr));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_agg_t<<<L.blocks_for(n * (kThreads / 64)), kThreads, 0, L.stream>>>(n, S, W.At, dZ, dHp);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     float* t = dH;
     dH = dHp;
     dHp = t;
   }
-  const int wi = kFeat * kHid + kHid;
-  (*L.counter) += 1;
-  k_in_bwd<<<gt, kThreads, 0, L.stream>>>(n, dH, H[0], F, part);
-  return reduce_parts(L, gt, wi, wi, part, grad, nullptr);
+  (*L.counter) += 2;
+  k_in_bwd<<<gt, kThreads, 0, L.stream>>>(n, dH, H[0], F, add(gt, wi, wi, grad, nullptr));
+  k_reduce_parts<<<blocks, kThreads, 0, L.stream>>>(PL);
+  return cudaGetLastError();
 }
 
 cudaError_t mpnn_adam(const Launch& L, float* w, const float* g, float* m, float* v, float lr,
