@@ -154,7 +154,11 @@ typedef struct gspm_options {
   int ordering;       /* GSPM_ORDER_*                                                          */
   double dt;          /* time step, s (Delta tau = gamma0 m_s dt)                              */
   double alpha;       /* damping constant                                                       */
-  double rtol_gs;     /* relative residual targets of the three CG families (Sec. 3.1: 1e-7) */
+  /* relative residual targets of the three CG families (Sec. 3.1: 1e-7).  GSPM_PREC_F64 with a target
+   * above 1e-10 (the largest of the three in a step, its own in gspm_solve_elastic) uses one fixed
+   * order of operations at every size; at 1e-10 and below, and in GSPM_PREC_MIXED, faster forms whose
+   * sums round differently: CG solutions agree within their target, not within rounding.  */
+  double rtol_gs;
   double rtol_ms;
   double rtol_mech;
   int max_iter;       /* per CG solve; exceeding it returns GSPM_ENOCONV                       */
@@ -485,7 +489,8 @@ GSPM_API int gspm_mpnn_train(struct gspm_ctx* ctx, int iterations, double lr, ui
 /* ---- measurement ------------------------------------------------------------------------ */
 
 /* kernel classes for gspm_profile_*.  Where a solve's whole CG loop runs as one kernel (meshes up to
- * 400,000 nodes, FP64 280,000, batches 400,000), that launch counts as the class of its product. */
+ * 400,000 nodes, FP64 280,000, batches 400,000; FP64 at targets up to 1e-10 only), that launch counts
+ * as the class of its product. */
 #define GSPM_KCLASS_SPMV_MECH 0  /* 3x3-block SpMV + fused p.q of the mechanical CG (K^mech)  */
 #define GSPM_KCLASS_SPMV_GS 1    /* scalar multi-RHS SpMV + p.q of the GSPM CG solves         */
 #define GSPM_KCLASS_SPMV_MS 2    /* scalar SpMV + p.q of the magnetostatic CG (K^ms)          */

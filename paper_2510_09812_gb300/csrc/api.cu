@@ -192,6 +192,8 @@ class Engine final : public EngineBase {
       std::vector<double> k6;
       kb_ = host_symmetric_blocks(hs, ops.Kmech, &k6) ? 6 : 9;
       ST(upload(&Kmech_, kb_ == 6 ? k6 : ops.Kmech));
+      // (the stored mean of A_ab and A_ba differs in its last bit from both)
+      if (!kRounded && kb_ == 6) ST(upload(&Kmech9_, ops.Kmech));
     }
     // inverse diagonals of M + eps K and M + alpha eps K (Jacobi preconditioner of the GSPM
     // solves): a row's diagonal is the sum of its entries in its own column (SELL padding
@@ -369,12 +371,16 @@ class Engine final : public EngineBase {
       *ms /= 5.f;
       return GSPM_OK;
     };
-    float best_b = 1e30f, best_s = 1e30f, best_g = 1e30f;
+    float best_b = 1e30f, best_9 = 1e30f, best_s = 1e30f, best_g = 1e30f;
     for (int v = 0; v < kSpmvVariants; ++v) {
       float t = 0.f;
       ST(time_variant(Kmech_, kb_, 1, 1, pinned, v, &t));
-      tune_ms_block_[v] = t;
       if (t < best_b) { best_b = t; var_block_ = v; }
+      if (Kmech9_) {
+        ST(time_variant(Kmech9_, 9, 1, 1, pinned, v, &t));
+        if (t < best_9) { best_9 = t; var_block9_ = v; }
+      }
+      tune_ms_block_[v] = t;
       ST(time_variant(Kms_, 1, 1, 1, pinned, v, &t));
       tune_ms_scalar_[v] = t;
       if (t < best_s) { best_s = t; var_scalar_ = v; }
@@ -395,7 +401,7 @@ class Engine final : public EngineBase {
  public:
   void tune_info(int* vb, int* vs, int* vg, float* tb, float* ts, float* tg,
                  int* item_slices) const override {
-    *vb = var_block_;
+    *vb = Kmech9_ ? var_block9_ : var_block_;
     *vs = var_scalar_;
     *vg = var_gs_;
     *item_slices = item_slices_;
@@ -456,7 +462,8 @@ class Engine final : public EngineBase {
                        L_.stream));
     CK(cudaMemsetAsync(bad_, 0, nseg_ * sizeof(int), L_.stream));
     const bool graph = graph_on_ && prof_mask_ == 0;
-    if (graph || loop_on_) {
+    set_fast(std::max(opt_.rtol_gs, std::max(opt_.rtol_ms, opt_.rtol_mech)));
+    if (graph || loop_now()) {
       const int rc = step_device(n_steps, D, printed, st, graph);
       if (rc != GSPM_OK && rc != GSPM_ENOCONV) return rc;
       ST(check_finite());
@@ -572,7 +579,7 @@ class Engine final : public EngineBase {
     // a6 b^mech = F^mech E0, a7 CG on pinned K^mech, x0 per the initial-guess mode
     TK(GSPM_KCLASS_RHS_MECH, launch_gdiv<T>(L_, A_, SG_, G_, sig0_, b_, pinned_));
     ST(mech_initial_guess(m_, x0_mode_));
-    ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, opt_.rtol_mech, &si->imech));
+    ST(solve_system(kSlotMech, kmech(), kb(), b_, u_, ulo_, opt_.rtol_mech, &si->imech));
     // a8 strain E = E_bar + sym grad u
     TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     // a9 h(m^n)
@@ -608,7 +615,7 @@ class Engine final : public EngineBase {
       TK(GSPM_KCLASS_POINTWISE, launch_e0<T>(L_, n, ms_, ld, mag_, D, E0_, sig0_));
       TK(GSPM_KCLASS_POINTWISE, launch_wsum<T>(L_, SG_, 6, E0_, ld, 1, w_, ebar(), eext(), red_));
       TK(GSPM_KCLASS_RHS_MECH, launch_gdiv<T>(L_, A_, SG_, G_, sig0_, b_, pinned_));
-      ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, opt_.rtol_mech, &si->imech2));
+      ST(solve_system(kSlotMech, kmech(), kb(), b_, u_, ulo_, opt_.rtol_mech, &si->imech2));
       TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     }
     TK(GSPM_KCLASS_POINTWISE, launch_hfield<T>(L_, n, SG_, ms_, hd_, E_, ld, mbar_s(), hz(), mag_, D, 1, P_.alpha * P_.dtau, nullptr, x_));
@@ -889,10 +896,12 @@ class Engine final : public EngineBase {
     TK(GSPM_KCLASS_POINTWISE, launch_wsum<T>(L_, SG_, 6, E0_, ld, 1, w_, ebar(), eext(), red_));
     TK(GSPM_KCLASS_RHS_MECH, launch_gdiv<T>(L_, A_, SG_, G_, sig0_, b_, pinned_));
     std::vector<SolveInfo> info;
-    ST(solve_system(kSlotMech, Kmech_, kb_, b_, u_, ulo_, rtol > 0 ? rtol : opt_.rtol_mech, &info));
+    if (!(rtol > 0)) rtol = opt_.rtol_mech;
+    set_fast(rtol);
+    ST(solve_system(kSlotMech, kmech(), kb(), b_, u_, ulo_, rtol, &info));
     TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     if (u) ST(export_field(u_, 1, 3, 3, u, where, ulo_));
-    if (loop_on_) ST(read_mech_info(&info));
+    if (loop_now()) ST(read_mech_info(&info));
     CK(cudaStreamSynchronize(L_.stream));
     int it = 0, nc = 0;
     double rel = 0.0;
@@ -946,7 +955,8 @@ class Engine final : public EngineBase {
       case GSPM_OP_K_MECH:
         ST(import_field(x, where, 3, tin_, 1, 3, nullptr));
         ST(pin_hide(3));
-        CK(launch_spmv<T>(L_, A_, Kmech_, kb_, tin_, tout_, var_block_, 1));
+        if (Kmech9_) CK(launch_spmv<T>(L_, A_, Kmech9_, 9, tin_, tout_, var_block9_, 1));
+        else CK(launch_spmv<T>(L_, A_, Kmech_, kb_, tin_, tout_, var_block_, 1));
         ST(pin_restore(3));
         ST(export_field(tout_, 1, 3, 3, y, where));
         break;
@@ -1324,7 +1334,22 @@ class Engine final : public EngineBase {
     return GSPM_OK;
   }
 
-  // K x = b for one K^ms (B = 1) or K^mech (B = kb_) solve.  Mixed precision: iterative
+  // Two CG runs on one system whose sums differ in rounding only agree within a good part of their
+  // stopping tolerance, not within rounding: orthogonality is lost on the way, and a residual near
+  // the tolerance may end a run one iteration earlier.  FP64 solutions (2-norm, relative) of the fused
+  // loops against the separate kernels: up to 2.8e-8 at 1e-7, 5.9e-9 at 1e-8, 1.0e-9 at 1e-9, 5e-11 at
+  // 1e-10.  So an FP64 call whose solves stop above kFastRtol keeps one arithmetic at every size: the
+  // separate kernels with z stored, nine values per block and the sums of seg_reduce_fixed.  Tighter
+  // ones, and all of mixed precision (whose results are held in FP32), take the fast forms.
+  static constexpr double kFastRtol = 1e-10;
+  static constexpr bool kRounded = sizeof(T) == 4;
+  void set_fast(double rtol) { fast_ = kRounded || rtol <= kFastRtol; }
+  bool loop_now() const { return loop_on_ && fast_; }
+  const T* kmech() const { return !fast_ && Kmech9_ ? Kmech9_ : Kmech_; }
+  int kb() const { return !fast_ && Kmech9_ ? 9 : kb_; }
+  int var_block() const { return !fast_ && Kmech9_ ? var_block9_ : var_block_; }
+
+  // K x = b for one K^ms (B = 1) or K^mech (B = kb()) solve.  Mixed precision: iterative
   // refinement (Wilkinson's scheme with the working-precision solver run in FP32): a first FP32
   // CG solve to kRtolInner leaves x; a second CG restarts from x, its initial residual b - K x
   // formed to twice the working precision (k_cg_init), and accumulates the correction in the
@@ -1347,7 +1372,7 @@ class Engine final : public EngineBase {
       CK(cudaMemsetAsync(dx_, 0, len * sizeof(T), L_.stream));
       ST(solve_general(slot2, val, B, b, x, dx_, rtol, &i2));
       TK(GSPM_KCLASS_CG_INIT, launch_refine_add<T>(L_, len, x, xlo, dx_));
-      if (!capturing_ && !loop_on_) {
+      if (!capturing_ && !loop_now()) {
         info->assign(nseg_, SolveInfo());
         for (int sg = 0; sg < nseg_; ++sg) {
           (*info)[sg].iters = i1[sg].iters + i2[sg].iters;
@@ -1361,7 +1386,7 @@ class Engine final : public EngineBase {
     return GSPM_OK;
   }
 
-  // CG for K x = b (B = 1 scalar K^ms, B = kb_ block K^mech), pinned or singular form, started from
+  // CG for K x = b (B = 1 scalar K^ms, B = kb() block K^mech), pinned or singular form, started from
   // x0 (read only) with the iterates accumulated into x: x == x0 is the plain solve; x != x0
   // (zero on entry) is the correction solve of solve_system, whose solution is x0 + x
   int solve_general(int slot, const T* val, int B, const T* b, const T* x0, T* x, double rtol,
@@ -1400,7 +1425,7 @@ class Engine final : public EngineBase {
       return GSPM_OK;
     };
     TK(GSPM_KCLASS_CG_INIT, launch_cg_init<T>(L_, A_, SG_, val, B, b, x0, r_, p_, st, na, rtol, opt_.max_iter, red_, pinned_ ? nullptr : bmean, pinned_, pc ? 1 : 0));
-    if (loop_on_) {
+    if (loop_now()) {
       if (!pinned_ && !pc) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
       CgLoop<T> a = loop_args(slot, val, len, x, dinv, B == 1 ? 0 : 1);
       a.pinned = pinned_;
@@ -1411,7 +1436,7 @@ class Engine final : public EngineBase {
       return GSPM_OK;
     }
     // aggregates that are runs of rows: z is never stored (see launch_pcg_update)
-    const bool runs = pc && pieces_ok_;
+    const bool runs = pc && pieces_ok_ && fast_;
     auto coarse = [&](int first) -> int {
       TK(GSPM_KCLASS_CG_VEC, launch_pcg_update<T>(L_, SG_, PP_, epr, r_, q_, dinv, pieces_, st, na, first, red_));
       TK(GSPM_KCLASS_CG_VEC, launch_pcg_coarse<T>(L_, SG_, CC_, PP_, TL, epr == 3 ? crows3_ : crows1_, epr, cinv, rco, pieces_, rc_, qsym_, ec_, st, first, red_));
@@ -1426,7 +1451,7 @@ class Engine final : public EngineBase {
       if (!pinned_) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
     }
     auto iter = [&]() -> int {
-      TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_spmv<T>(L_, A_, SG_, val, B, 1, len, p_, q_, st, red_, B == 1 ? var_scalar_ : var_block_, pinned_, 1));
+      TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_spmv<T>(L_, A_, SG_, val, B, 1, len, p_, q_, st, red_, B == 1 ? var_scalar_ : var_block(), pinned_, 1));
       if (runs) {
         ST(coarse(0));
         TK(GSPM_KCLASS_CG_VEC, launch_pcg_p<T>(L_, SG_, CC_, epr, r_, dinv, ec_, p_, x, st, loop_, 0));
@@ -1462,7 +1487,7 @@ class Engine final : public EngineBase {
     CK(cudaMemsetAsync(na, 0, sizeof(int), L_.stream));
     const T* dinv = aval == Aeps_ ? dgs_eps_ : dgs_aeps_;  // NULL: plain CG
     TK(GSPM_KCLASS_CG_INIT, launch_cg_init_gs<T>(L_, A_, SG_, aval, M_, nr, ld_, x, r_, p_, st, na, opt_.rtol_gs, opt_.max_iter, red_, dinv));
-    if (loop_on_) {
+    if (loop_now()) {
       CgLoop<T> a = loop_args(slot, aval, ld_, x, dinv, 2);
       const int npc = dinv ? 2 : 0;
       a.place = loop_place(1, nr, npc);
@@ -2168,6 +2193,7 @@ class Engine final : public EngineBase {
   Launch L_;
   DevMem mem_;
   int kb_ = 9;  // stored values per K^mech block: 6 (symmetric) or 9
+  bool fast_ = false;  // of the current call, see set_fast
   int64_t n_ = 0, ld_ = 0, nslices_ = 0, entries_ = 0, nmag_ = 0, nodes_ = 0;
   int nseg_ = 1, nitems_ = 0, item_slices_ = 1;
   DSeg SG_{};
@@ -2179,7 +2205,7 @@ class Engine final : public EngineBase {
   int32_t* slen_ = nullptr;
   int32_t* col_ = nullptr;
   T *Kms_ = nullptr, *Aeps_ = nullptr, *Aaeps_ = nullptr, *M_ = nullptr, *F_ = nullptr,
-    *G_ = nullptr, *Kmech_ = nullptr;
+    *G_ = nullptr, *Kmech_ = nullptr, *Kmech9_ = nullptr;
   double *invML_ = nullptr, *w_ = nullptr;
   uint8_t* mag_ = nullptr;
   int64_t* perm_ = nullptr;
@@ -2192,7 +2218,7 @@ class Engine final : public EngineBase {
   CGState* host_state_ = nullptr;
   Red red_{};
   int pred_[kSolveSlots];
-  int var_block_ = 0, var_scalar_ = 0, var_gs_ = 0;
+  int var_block_ = 0, var_block9_ = 0, var_scalar_ = 0, var_gs_ = 0;
   float tune_ms_block_[kSpmvVariants] = {}, tune_ms_scalar_[kSpmvVariants] = {},
         tune_ms_gs_[kSpmvVariants] = {};
   int seen_[kSolveSlots] = {};

@@ -75,7 +75,8 @@ __host__ __device__ constexpr int pow2_up(int n) { return n <= 1 ? 1 : 2 * pow2_
 // Sums of M values (a power of two) over each group of LANES lanes.  While several values are
 // left, a pair of lanes splits them: each keeps half of them and adds the other lane's, so M
 // values take M - 1 + log2(LANES / M) additions where M separate trees take M log2(LANES).  The
-// result is value (lane % LANES) / (LANES / M), the same bits in every lane that has it.
+// result is value (lane % LANES) / (LANES / M), the same bits in every lane that has it: those of a
+// tree per value with halving distances.
 template <int M, int LANES, typename V>
 __device__ __forceinline__ V lane_sums(V (&v)[M]) {
   const int lane = threadIdx.x & 31;
@@ -93,6 +94,35 @@ __device__ __forceinline__ V lane_sums(V (&v)[M]) {
 #pragma unroll
   for (int r = LANES / M; r > 1; r >>= 1) v[0] = plus(v[0], lane_xor(v[0], r / 2));
   return v[0];
+}
+
+// The same with doubling distances (the bits of a tree per value that starts with neighbours): the
+// result is value lane % M with its bits in reverse order.
+template <int M, int LANES, typename V>
+__device__ __forceinline__ V lane_sums_up(V (&v)[M]) {
+  const int lane = threadIdx.x & 31;
+  int o = 1;
+#pragma unroll
+  for (int w = M / 2; w >= 1; w >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const V send = up ? v[i] : v[i + w];
+      v[i] = plus(up ? v[i + w] : v[i], lane_xor(send, o));
+    }
+    o <<= 1;
+  }
+#pragma unroll
+  for (; o < LANES; o <<= 1) v[0] = plus(v[0], lane_xor(v[0], o));
+  return v[0];
+}
+// lane % M with its bits in reverse order
+template <int M>
+__device__ __forceinline__ int lane_value_up(int lane) {
+  int k = 0;
+#pragma unroll
+  for (int w = M / 2, o = 1; w >= 1; w >>= 1, o <<= 1) k += lane & o ? w : 0;
+  return k;
 }
 
 // The last item of `seg` to arrive (its block partials, a row of pow2_up(NC) values, already in
@@ -176,14 +206,78 @@ __device__ __forceinline__ bool seg_reduce_of(V (&v)[pow2_up(NC)], int item, int
   return seg_arrive<NC>(item, seg, G, IL, red, res);
 }
 
-// the same for FP64 values
+// Sum over a warp's lanes, distances halving; the result is lane 0's
+__device__ __forceinline__ double warp_sum(double x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
+  return x;
+}
+
+// The reduction of FP64 contexts: one tree of 32 lanes and one of the warps per value, then the item
+// partials strided over the block's threads and the same trees.  A CG solve in FP64 that stops at a
+// loose tolerance magnifies the rounding of its sums (1e-16) to 1e-9 .. 1e-8 of the solution, so this
+// order of additions is part of what such a context returns and does not follow the faster one above.
 template <int NC>
+__device__ __forceinline__ bool seg_reduce_fixed(double (&v)[NC], int item, int seg, const DSeg& G,
+                                                 const ItemList& IL, const Red& red, double* res) {
+  __shared__ double sm[NC][32];
+  __shared__ int am_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const double x = warp_sum(v[c]);
+    if (lane == 0) sm[c][warp] = x;
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const double x = warp_sum(lane < nw ? sm[c][lane] : 0.0);
+      if (lane == 0) red.partial[(int64_t)item * kRedComp + c] = x;
+    }
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(G.counter + seg, 1u);
+    am_last = (t == (unsigned)IL.seg_nitems[seg] - 1u);
+  }
+  __syncthreads();
+  if (!am_last) return false;
+  __threadfence();
+  const int i0 = IL.seg_item0[seg], ni = IL.seg_nitems[seg];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    double acc = 0.0;
+    for (int b = threadIdx.x; b < ni; b += blockDim.x)
+      acc += __ldcg(red.partial + (int64_t)(i0 + b) * kRedComp + c);
+    acc = warp_sum(acc);
+    if (lane == 0) sm[c][warp] = acc;
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const double x = warp_sum(lane < nw ? sm[c][lane] : 0.0);
+      if (lane == 0) res[c] = x;
+    }
+  }
+  if (threadIdx.x == 0) G.counter[seg] = 0u;
+  __syncthreads();
+  return true;
+}
+
+// FP64 values in a context of working precision T
+template <typename T, int NC>
 __device__ __forceinline__ bool seg_reduce(double (&v)[NC], int item, int seg, const DSeg& G,
                                            const ItemList& IL, const Red& red, double* res) {
-  double x[pow2_up(NC)];
+  if constexpr (std::is_same<T, double>::value) {
+    return seg_reduce_fixed<NC>(v, item, seg, G, IL, red, res);
+  } else {
+    double x[pow2_up(NC)];
 #pragma unroll
-  for (int c = 0; c < pow2_up(NC); ++c) x[c] = c < NC ? v[c < NC ? c : 0] : 0.0;
-  return seg_reduce_of<NC>(x, item, seg, G, IL, red, res);
+    for (int c = 0; c < pow2_up(NC); ++c) x[c] = c < NC ? v[c < NC ? c : 0] : 0.0;
+    return seg_reduce_of<NC>(x, item, seg, G, IL, red, res);
+  }
 }
 
 // seg_reduce of per-thread values given as unevaluated sums hi + lo in T.  T = float: the warp
@@ -198,7 +292,7 @@ __device__ __forceinline__ bool seg_reduce_hl(const T (&hi)[NC], const T (&lo)[N
     double v[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) v[c] = hi[c] + lo[c];
-    return seg_reduce<NC>(v, item, seg, G, IL, red, res);
+    return seg_reduce<T, NC>(v, item, seg, G, IL, red, res);
   } else {
     DF x[pow2_up(NC)];
 #pragma unroll

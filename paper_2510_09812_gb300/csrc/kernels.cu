@@ -29,8 +29,9 @@ namespace {
 // volume average per segment: out[seg*NC + c] = sum_i w_i f(i, c) (+ add[c]); Sec. 2.4 with
 // nodal weights M_L,i / V(segment)
 // ------------------------------------------------------------------------------------------
+// NC: components, FP64 contexts 9 with nc of them used (see seg_reduce_fixed)
 template <typename T, int NC>
-__global__ void __launch_bounds__(kBlock) k_wsum(DSeg G, ItemList IL, const T* __restrict__ f,
+__global__ void __launch_bounds__(kBlock) k_wsum(DSeg G, ItemList IL, int nc, const T* __restrict__ f,
                                                  int64_t cs, int64_t ns,
                                                  const double* __restrict__ w, double* out,
                                                  const double* add, Red red) {
@@ -44,11 +45,12 @@ __global__ void __launch_bounds__(kBlock) k_wsum(DSeg G, ItemList IL, const T* _
       if (!row_valid(G, seg, i)) continue;
       const double wi = w[i];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) v[c] += wi * (double)f[i * ns + c * cs];
+      for (int c = 0; c < NC; ++c)
+        if (NC < 9 || c < nc) v[c] += wi * (double)f[i * ns + c * cs];
     }
     __shared__ double res[NC];
-    if (seg_reduce<NC>(v, item, seg, G, IL, red, res) && threadIdx.x == 0)
-      for (int c = 0; c < NC; ++c) out[seg * NC + c] = res[c] + (add ? add[c] : 0.0);
+    if (seg_reduce<T, NC>(v, item, seg, G, IL, red, res) && threadIdx.x == 0)
+      for (int c = 0; c < nc; ++c) out[seg * nc + c] = res[c] + (add ? add[c] : 0.0);
   }
 }
 
@@ -218,7 +220,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_init(DSell A, DSeg G, ItemList IL
       }
     }
     __shared__ double res[2 + NC];
-    if (seg_reduce<2 + NC>(v, item, seg, G, IL, red, res) && threadIdx.x == 0) {
+    if (seg_reduce<T, 2 + NC>(v, item, seg, G, IL, red, res) && threadIdx.x == 0) {
       // projected form: r.r without the constant part of r, p0 = r0 minus its mean
       const double inv_n = 1.0 / (double)G.seg_nrow[seg];
       double s2 = 0.0;
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_init_gs(DSell A, DSeg G, ItemList
       }
     }
     __shared__ double res[3 * NR];
-    if (seg_reduce<3 * NR>(v, item, seg, G, IL, red, res) && threadIdx.x == 0) {
+    if (seg_reduce<T, 3 * NR>(v, item, seg, G, IL, red, res) && threadIdx.x == 0) {
       double bb[NR], rr[NR], rz[NR];
       for (int k = 0; k < NR; ++k) {
         rr[k] = res[3 * k];
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(kBlock) k_true_res(DSell A, DSeg G, ItemList I
       }
     }
     __shared__ double res[2];
-    if (seg_reduce<2>(v, item, seg, G, IL, red, res) && threadIdx.x == 0) {
+    if (seg_reduce<T, 2>(v, item, seg, G, IL, red, res) && threadIdx.x == 0) {
       out[2 * seg] = res[0];
       out[2 * seg + 1] = res[1];
     }
@@ -766,6 +768,82 @@ __global__ void __launch_bounds__(kBlock) k_restrict(DCoarse C, const T* __restr
 }
 
 
+// The same for contiguous aggregates (GSPM_ORDER_AGGREGATE) of scalar rows: one warp per
+// aggregate, no barrier.  The aggregate's elements [e0, e1) of r are read as 16-byte packs, kRestrictPacks per
+// lane in flight, with the unaligned head and tail (fewer than one pack each) taken by single
+// lanes; element e has component e mod EPR.  Each lane sums its packs in order, the warp tree is
+// fixed, so the result does not depend on the grid.
+constexpr int kRestrictPacks = 8;
+template <typename T, int EPR>
+__global__ void __launch_bounds__(kBlock) k_restrict_contig(DCoarse C, const T* __restrict__ r,
+                                                            const int64_t* __restrict__ rc_off,
+                                                            T* __restrict__ rc) {
+  pdl_enter();
+  constexpr int W = Pack16<T>::W, U = kRestrictPacks;
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t I = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; I < C.nagg;
+       I += nwarps) {
+    const int q0 = C.agg_ptr[I], q1 = C.agg_ptr[I + 1];
+    T acc[EPR];
+#pragma unroll
+    for (int a = 0; a < EPR; ++a) acc[a] = T(0);
+    if (q1 > q0) {
+      const int64_t e0 = (int64_t)C.agg_rows[q0] * EPR, e1 = e0 + (int64_t)(q1 - q0) * EPR;
+      int64_t a0 = (e0 + W - 1) / W * W;
+      if (a0 > e1) a0 = e1;
+      int64_t a1 = e1 / W * W;
+      if (a1 < a0) a1 = a0;
+      const int nh = (int)(a0 - e0), nt = (int)(e1 - a1);
+      if (lane < nh + nt) {
+        const int64_t e = lane < nh ? e0 + lane : a1 + (lane - nh);
+        acc[EPR == 1 ? 0 : (int)(e % EPR)] += r[e];
+      }
+      const int64_t np = (a1 - a0) / W;
+      const int cb0 = EPR == 1 ? 0 : (int)(a0 % EPR);
+      for (int64_t t0 = 0; t0 < np; t0 += 32 * U) {
+        T v[U][W];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t t = t0 + 32 * u + lane;
+          if (t < np) {
+            ld16(r + a0 + t * W, v[u]);
+          } else {
+#pragma unroll
+            for (int c = 0; c < W; ++c) v[u][c] = T(0);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t t = t0 + 32 * u + lane;
+          // component of the pack's first element: (a0 + t W) mod EPR
+          const int cb = EPR == 1 ? 0 : (int)((cb0 + (t % EPR) * (W % EPR)) % EPR);
+#pragma unroll
+          for (int c = 0; c < W; ++c) {
+            if (EPR == 1) {
+              acc[0] += v[u][c];
+            } else {
+              const int cc = (cb + c) % EPR;
+#pragma unroll
+              for (int a = 0; a < EPR; ++a) acc[a] += cc == a ? v[u][c] : T(0);
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < EPR; ++a) {
+      T v = acc[a];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
+      if (lane == 0) {
+        const int sg = C.agg_seg[I];
+        rc[rc_off[sg] + (I - C.seg_agg0[sg]) * EPR + a] = v;
+      }
+    }
+  }
+}
+
 // N contiguous values through 16-byte packs (N * sizeof(T) a multiple of 16, p aligned)
 template <typename T, int N>
 __device__ __forceinline__ void ldn(const T* p, T (&v)[N]) {
@@ -869,9 +947,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_coarse_symv_tiles(DSymTiles TL,
         cs[c] += w[c] * xi;
       }
     }
-    const T row_sum = lane_sums<NP, LPR>(rs);
-    if (cp % (LPR / NP) == 0)
-      srow[set][cp / (LPR / NP) * RPP + warp * RPW + rg] = row_sum;
+    const T row_sum = lane_sums_up<NP, LPR>(rs);
+    if (cp < NP) srow[set][lane_value_up<NP>(cp) * RPP + warp * RPW + rg] = row_sum;
 #pragma unroll
     for (int o = LPR; o < 32; o <<= 1)
 #pragma unroll
@@ -896,23 +973,32 @@ __global__ void __launch_bounds__(kBlock, 4) k_coarse_symv_tiles(DSymTiles TL,
 }
 
 // Sum over the tile columns of 32 coarse rows of Q (group grp of the segment), a warp's lanes on
-// the rows and the block's warps on the columns, in a fixed order: valid in warp 0, a row per lane
+// the rows and the block's warps on the columns: valid in warp 0, a row per lane.  The order of the
+// additions is that of a warp per row, its lanes on the columns (32 running sums, then a tree with
+// halving distances): warp w keeps the sums w, w + 8, w + 16 and w + 24.
 template <typename T>
 __device__ __forceinline__ T coarse_rows_sum(const T* __restrict__ q, int64_t Tn, int64_t grp,
                                              T (&sm)[kBlock / 32][32]) {
   constexpr int TS = coarse_tile<T>(), NW = kBlock / 32, GP = TS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const T* p = q + (grp / GP) * Tn * TS + (grp % GP) * 32 + lane;
-  T acc = T(0);
-#pragma unroll 4
-  for (int64_t J = warp; J < Tn; J += NW) acc += p[J * TS];
-  sm[warp][lane] = acc;
-  __syncthreads();
-  T v = T(0);
-  if (warp == 0)
+  static_assert(NW == 8, "four sums per warp");
+  T acc[4] = {T(0), T(0), T(0), T(0)};
+  for (int64_t J = warp; J < Tn; J += 4 * NW)
 #pragma unroll
-    for (int w = 0; w < NW; ++w) v += sm[w][lane];
-  return v;
+    for (int u = 0; u < 4; ++u)
+      if (J + u * NW < Tn) acc[u] += p[(J + u * NW) * TS];
+  sm[warp][lane] = (acc[0] + acc[2]) + (acc[1] + acc[3]);
+  __syncthreads();
+  if (warp) return T(0);
+  T v[NW];
+#pragma unroll
+  for (int w = 0; w < NW; ++w) v[w] = sm[w][lane];
+#pragma unroll
+  for (int h = NW / 2; h >= 1; h >>= 1)
+#pragma unroll
+    for (int w = 0; w < h; ++w) v[w] += v[w + h];
+  return v[0];
 }
 
 // ec = the row sums of Q; items: groups of 32 coarse rows of a segment
@@ -1853,7 +1939,7 @@ __global__ void __launch_bounds__(kBlock) k_project(DSeg G, ItemList IL, int64_t
       m[2 * ld + i] = nc;
     }
     __shared__ double res[1];
-    if (seg_reduce<1>(v, item, seg, G, IL, red, res) && threadIdx.x == 0)
+    if (seg_reduce<T, 1>(v, item, seg, G, IL, red, res) && threadIdx.x == 0)
       dm_out[seg] = res[0] * inv_nmag[seg];
   }
 }
@@ -1949,8 +2035,10 @@ struct ItemGrid {
   int grid;
   ItemList list;
 };
-static ItemGrid item_grid(const Launch& L, const DSeg& G, const void* kernel) {
-  const int per_sm = resident_per_sm(kernel);
+// blocks > 0 names the list instead: FP64 contexts do, whose results the division into items is part
+// of (see seg_reduce_fixed); the numbers are the residencies that the kernels had when this was fixed.
+static ItemGrid item_grid(const Launch& L, const DSeg& G, const void* kernel, int blocks = 0) {
+  const int per_sm = blocks ? blocks : resident_per_sm(kernel);
   const ItemList& il = G.list[(per_sm < kItemLists ? per_sm : kItemLists) - 1];
   return ItemGrid{grid_for(L, (int64_t)il.nitems * kBlock, kernel), il};
 }
@@ -1984,13 +2072,16 @@ static cudaError_t launch_pdl(void (*k)(KArgs...), int grid, cudaStream_t stream
 
 #define GSPM_GRID(L, threads, kern) grid_for((L), (threads), reinterpret_cast<const void*>(kern))
 #define GSPM_IGRID(L, G, kern) item_grid((L), (G), reinterpret_cast<const void*>(kern))
+#define GSPM_IGRID64(L, G, kern, blocks)                    \
+  item_grid((L), (G), reinterpret_cast<const void*>(kern), \
+            std::is_same<T, double>::value ? (blocks) : 0)
 
 template <typename T, int NC>
-static cudaError_t wsum_nc(const Launch& L, const DSeg& G, const T* f, int64_t cs, int64_t ns,
+static cudaError_t wsum_nc(const Launch& L, const DSeg& G, int nc, const T* f, int64_t cs, int64_t ns,
                            const double* w, double* out, const double* add, Red red) {
   auto k = k_wsum<T, NC>;
-  const ItemGrid ig = GSPM_IGRID(L, G, k);
-  k<<<ig.grid, kBlock, 0, L.stream>>>(G, ig.list, f, cs, ns, w, out, add, red);
+  const ItemGrid ig = GSPM_IGRID64(L, G, k, 5);
+  k<<<ig.grid, kBlock, 0, L.stream>>>(G, ig.list, nc, f, cs, ns, w, out, add, red);
   return cudaGetLastError();
 }
 
@@ -1998,12 +2089,16 @@ template <typename T>
 cudaError_t launch_wsum(const Launch& L, const DSeg& G, int nc, const T* f, int64_t cs,
                         int64_t ns, const double* w, double* out, const double* add, Red red) {
   (*L.counter) += 1;
-  switch (nc) {
-    case 1: return wsum_nc<T, 1>(L, G, f, cs, ns, w, out, add, red);
-    case 3: return wsum_nc<T, 3>(L, G, f, cs, ns, w, out, add, red);
-    case 6: return wsum_nc<T, 6>(L, G, f, cs, ns, w, out, add, red);
+  if constexpr (std::is_same<T, double>::value) {
+    return wsum_nc<T, 9>(L, G, nc, f, cs, ns, w, out, add, red);
+  } else {
+    switch (nc) {
+      case 1: return wsum_nc<T, 1>(L, G, nc, f, cs, ns, w, out, add, red);
+      case 3: return wsum_nc<T, 3>(L, G, nc, f, cs, ns, w, out, add, red);
+      case 6: return wsum_nc<T, 6>(L, G, nc, f, cs, ns, w, out, add, red);
+    }
+    return cudaErrorInvalidValue;
   }
-  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_volume_avg(const Launch& L, int nseg, int64_t max_nodes, const int64_t* node0,
@@ -2052,17 +2147,17 @@ cudaError_t launch_cg_init(const Launch& L, const DSell& A, const DSeg& G, const
   (*L.counter) += 1;
   if (B == 1) {
     auto k = k_cg_init<T, 1>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, 5);
     k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, r, p, st, nactive, rtol,
                                         max_iter, red, bmean, pinned, pc);
   } else if (B == 6) {
     auto k = k_cg_init<T, 6>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, 4);
     k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, r, p, st, nactive, rtol,
                                         max_iter, red, bmean, pinned, pc);
   } else {
     auto k = k_cg_init<T, 9>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, 4);
     k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, val, b, x, r, p, st, nactive, rtol,
                                         max_iter, red, bmean, pinned, pc);
   }
@@ -2127,21 +2222,21 @@ cudaError_t launch_cg_init_gs(const Launch& L, const DSell& A, const DSeg& G, co
   switch (nr) {
     case 1: {
       auto k = k_cg_init_gs<T, 1>;
-      const ItemGrid ig = GSPM_IGRID(L, G, k);
+      const ItemGrid ig = GSPM_IGRID64(L, G, k, 5);
       k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, aval, mval, ld, x, r, p, st, nactive,
                                                       rtol, max_iter, red, dinv);
       break;
     }
     case 2: {
       auto k = k_cg_init_gs<T, 2>;
-      const ItemGrid ig = GSPM_IGRID(L, G, k);
+      const ItemGrid ig = GSPM_IGRID64(L, G, k, 5);
       k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, aval, mval, ld, x, r, p, st, nactive,
                                                       rtol, max_iter, red, dinv);
       break;
     }
     case 3: {
       auto k = k_cg_init_gs<T, 3>;
-      const ItemGrid ig = GSPM_IGRID(L, G, k);
+      const ItemGrid ig = GSPM_IGRID64(L, G, k, 4);
       k<<<ig.grid, kBlock, 0, L.stream>>>(A, G, ig.list, aval, mval, ld, x, r, p, st, nactive,
                                                       rtol, max_iter, red, dinv);
       break;
@@ -2151,6 +2246,14 @@ cudaError_t launch_cg_init_gs(const Launch& L, const DSell& A, const DSeg& G, co
   return cudaGetLastError();
 }
 
+// list of the FP64 products (see item_grid)
+template <int B, int NR, int VAR>
+static constexpr int spmv64_blocks() {
+  if (VAR == 3) return 3;
+  if (B == 9) return VAR == 1 ? 1 : 2;
+  if (NR == 1) return VAR == 1 ? 3 : 4;
+  return NR == 2 && VAR == 0 ? 3 : 2;
+}
 template <typename T, int VAR>
 static cudaError_t cg_spmv_variant(const Launch& L, const DSell& A, const DSeg& G, const T* val,
                                    int B, int nr, int64_t ld, const T* p, T* q, CGState* st,
@@ -2161,7 +2264,7 @@ static cudaError_t cg_spmv_variant(const Launch& L, const DSell& A, const DSeg& 
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
   } else if (B == 9) {
     auto k = k_cg_spmv<T, 9, 1, VAR, kDiff<T>>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, (spmv64_blocks<9, 1, VAR>()));
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
   } else if (nr == 1 && diff && kDiff<T>) {
     auto k = k_cg_spmv<T, 1, 1, VAR, 1>;
@@ -2169,15 +2272,15 @@ static cudaError_t cg_spmv_variant(const Launch& L, const DSell& A, const DSeg& 
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
   } else if (nr == 1) {
     auto k = k_cg_spmv<T, 1, 1, VAR, 0>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, (spmv64_blocks<1, 1, VAR>()));
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
   } else if (nr == 2) {
     auto k = k_cg_spmv<T, 1, 2, VAR, 0>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, (spmv64_blocks<1, 2, VAR>()));
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
   } else if (nr == 3) {
     auto k = k_cg_spmv<T, 1, 3, VAR, 0>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, (spmv64_blocks<1, 3, VAR>()));
     return launch_pdl(k, ig.grid, L.stream, A, G, ig.list, val, ld, p, q, st, red, pinned);
   } else {
     return cudaErrorInvalidValue;
@@ -2204,7 +2307,7 @@ static cudaError_t cg_update_nr(const Launch& L, const DSeg& G, int epr, int64_t
                          const T* p, const T* q, CGState* st, int* nactive, Red red,
                          const T* dinv) {
   auto k = k_cg_update<T, NR, VEC>;
-  const ItemGrid ig = GSPM_IGRID(L, G, k);
+  const ItemGrid ig = GSPM_IGRID64(L, G, k, VEC ? (NR == 1 ? 4 : (NR == 2 ? 5 : 2)) : (NR == 1 ? 5 : 4));
   return launch_pdl(k, ig.grid, L.stream, G, ig.list, epr, ld, x, r, p, q, st, nactive, red, dinv);
 }
 
@@ -2270,7 +2373,12 @@ template <typename T>
 cudaError_t launch_restrict(const Launch& L, const DCoarse& C, int epr, const T* r,
                             const int64_t* rc_off, T* rc) {
   (*L.counter) += 1;
-  if (epr == 3) {
+  // scalar rows: a warp per contiguous aggregate (6.4 against 13 us per launch at 3M nodes,
+  // cold); three components: a block per aggregate (15.9 us against 23 us for a warp)
+  if (epr == 1 && C.contig && aligned16(r)) {
+    auto k = k_restrict_contig<T, 1>;
+    ST_CUDA(launch_pdl(k, GSPM_GRID(L, C.nagg * 32, k), L.stream, C, r, rc_off, rc));
+  } else if (epr == 3) {
     auto k = k_restrict<T, 3>;
     ST_CUDA(launch_pdl(k, GSPM_GRID(L, C.nagg * kBlock, k), L.stream, C, r, rc_off, rc));
   } else if (epr == 1) {
@@ -2378,11 +2486,11 @@ cudaError_t launch_pcg_z(const Launch& L, const DSeg& G, const DCoarse& C, int e
   (*L.counter) += 1;
   if (epr == 3) {
     auto k = k_pcg_z<T, 3>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, 3);
     ST_CUDA(launch_pdl(k, ig.grid, L.stream, G, ig.list, C, r, dinv, ec, z, st, init, red));
   } else if (epr == 1) {
     auto k = k_pcg_z<T, 1>;
-    const ItemGrid ig = GSPM_IGRID(L, G, k);
+    const ItemGrid ig = GSPM_IGRID64(L, G, k, 5);
     ST_CUDA(launch_pdl(k, ig.grid, L.stream, G, ig.list, C, r, dinv, ec, z, st, init, red));
   } else {
     return cudaErrorInvalidValue;
@@ -2523,7 +2631,7 @@ cudaError_t launch_project(const Launch& L, const DSeg& G, int64_t ld, const T* 
                            Red red, int* bad) {
   (*L.counter) += 1;
   auto k = k_project<T>;
-  const ItemGrid ig = GSPM_IGRID(L, G, k);
+  const ItemGrid ig = GSPM_IGRID64(L, G, k, 4);
   k<<<ig.grid, kBlock, 0, L.stream>>>(G, ig.list, ld, x, mag, m, dm_out, inv_nmag, red, bad);
   return cudaGetLastError();
 }
