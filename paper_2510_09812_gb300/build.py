@@ -37,7 +37,7 @@ def _sources():
     return [os.path.join(CSRC, s) for s in CUDA_SOURCES + CXX_SOURCES] + [
         os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "kernels.cuh"),
         os.path.join(CSRC, "device.cuh"),
-        os.path.join(CSRC, "flatsum.cuh"),
+        os.path.join(CSRC, "flatsum.cuh"), os.path.join(CSRC, "looplayout.h"),
         os.path.join(CSRC, "mpnn.cuh"),
         os.path.join(INCLUDE, "gspm.h")]
 

@@ -24,7 +24,8 @@
 // bounded: a block that gives up sets *err and returns, and so do the others after it.
 //
 // Meshes of a batch are independent groups of blocks: they neither wait for one another nor stop
-// together.
+// together.  Their exchange numbers drift apart, so their packets lie in ranges of their own
+// (looplayout.h; ex and line are per block).
 //
 // Measured (separate kernels -> fused): time steps at 1,024 nodes (FP64) 7.8 -> 3.1 ms, 19,305 nodes
 // (mixed) 14.8 -> 5.8, 65,536 (mixed) 18.4 -> 7.0, 65,536 hexahedra (FP64) 22.6 -> 12.6; an elastic
@@ -42,6 +43,7 @@
 
 #include "device.cuh"
 #include "kernels.cuh"
+#include "looplayout.h"
 
 namespace gspm {
 
@@ -384,12 +386,14 @@ template <> struct PWord<double> {
 };
 
 // Part of one SELL row's product with p, neighbours k0, k0 + ks, ...: a round's columns and values
-// are all loaded before its gathers.  p is read as packets of exchange ep; a lane past the
-// mesh's last row (not valid: its columns point at itself) reads none.  False: gave up.
+// are all loaded before its gathers.  p is read as packets of exchange ep (the mesh has m_rows rows
+// from m_row0, see looplayout.h); a lane past the mesh's last row (not valid: its columns point at
+// itself) reads none.  False: gave up.
 template <typename T, int B, int NR, bool DIFF>
 __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ val, int64_t s,
                                          int lane, const void* pp, uint32_t ep,
-                                         int64_t ld, const T (&xi)[B == 1 ? NR : 3], unsigned skip,
+                                         int64_t m_row0, int64_t m_rows,
+                                         const T (&xi)[B == 1 ? NR : 3], unsigned skip,
                                          bool valid, T (&acc)[B == 1 ? NR : 3], int k0, int ks) {
   constexpr int NV = B == 1 ? NR : 3;
   const int64_t base = A.sptr[s];
@@ -420,7 +424,7 @@ __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ v
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int c = 0; c < NV; ++c) {
-          const int64_t i = B == 1 ? c * ld + j[u] : 3 * (int64_t)j[u] + c;
+          const int64_t i = B == 1 ? p_packet1(m_row0, m_rows, j[u], c) : p_packet3(j[u], c);
           if (B != 1 || !(skip >> c & 1)) x[u][c] = PW::ld(pp, i);
         }
 #pragma unroll
@@ -511,6 +515,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   const bool leader = blk == b0;
   const int sl0 = P.sl0[blk], nsl = P.sl1[blk] - sl0;
   const int64_t row0 = (int64_t)sl0 * 32;
+  const int64_t m_row0 = (int64_t)P.sl0[b0] * 32, m_rows = (int64_t)P.sl1[b0 + nb - 1] * 32 - m_row0;
   const int64_t rend = a.G.seg_row0[seg] + a.G.seg_nrow[seg];
   const int64_t pin = a.pinned ? a.G.seg_pin[seg] : -1;
   uint32_t ep = P.epoch[2 * seg], bars = P.epoch[2 * seg + 1];
@@ -540,7 +545,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   const Rows<T, AOS> di = PC == 0 ? gd : place(4, const_cast<T*>(a.dinv));
   auto publish = [&](int c, int64_t lr, T v) {  // v is row lr's new p
     p.at(c, lr) = v;
-    put_p(P.pp, AOS ? 3 * (row0 + lr) + c : c * a.ld + row0 + lr, v, ep);
+    put_p(P.pp, AOS ? p_packet3(row0 + lr, c) : p_packet1(m_row0, m_rows, row0 + lr, c), v, ep);
   };
   ulonglong2* line = P.line + (int64_t)blk * 8;  // + kLn* * kLoopLines
 
@@ -635,8 +640,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
         T xi[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) xi[c] = DIFF && row0 + lr < rend ? p.at(c, lr) : T(0);
-        ok = ok && row_part<T, B, NR, DIFF>(a.A, a.val, sl0 + ls, lane, P.pp, ep, a.ld, xi, skip,
-                                            row0 + lr < rend, acc, k0, ks);
+        ok = ok && row_part<T, B, NR, DIFF>(a.A, a.val, sl0 + ls, lane, P.pp, ep, m_row0, m_rows, xi,
+                                            skip, row0 + lr < rend, acc, k0, ks);
       };
       if (split == 1) {
         for (int ls = warp; ls < nsl; ls += kNW) {
@@ -775,13 +780,13 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
         T v = T(0);
 #pragma unroll
         for (int w = 0; w < kNW; ++w) v += psum[((k / NC) * kNW + w) * NC + k % NC];
-        post(P.rcx + (int64_t)pc0 * NC + k, v, T(0), ep);
+        post(P.rcx + coarse_packet(segp0, pc0, NC, k), v, T(0), ep);
       }
     }
     if (PC == 1 && g1 > g0) {
       // server: its rows of the dense inverse times the restricted residual; r_c.e_c and the sums of
       // P e_c for the leader
-      if (!wait_coarse<T>(P.rcx + (int64_t)segp0 * NC, tid, kLoopThreads, segp * NC, ep, pieces))
+      if (!wait_coarse<T>(P.rcx + coarse_packet(segp0, segp0, NC, 0), tid, kLoopThreads, segp * NC, ep, pieces))
         s_fail = 1;
       __syncthreads();
       for (int k = tid; k < nagg * NC; k += kLoopThreads) {
@@ -805,7 +810,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
         for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(kFull, t, o);
         if (lane == 0) {
           // (read by the blocks of this aggregate's rows, which post their next pieces after it)
-          post(P.ecx + (int64_t)agg0 * NC + g, t, T(0), ep);
+          post(P.ecx + coarse_packet(agg0, agg0, NC, g), t, T(0), ep);
           const int I = agg0 + g / NC;
           const T cnt = (T)(a.C.agg_ptr[I + 1] - a.C.agg_ptr[I]);
           pair_add(ch[0], cl[0], t * rcs[g], T(0));
@@ -896,7 +901,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
       if (warp == 0)
         ok = wait_line(line + kLnBeta * kLoopLines, lane, LF::NB, ep, ln);
       else if (PC == 1)
-        ok = wait_coarse<T>(P.ecx + (int64_t)la0 * NC, tid - 32, kLoopThreads - 32, np * NC, ep, ecl);
+        ok = wait_coarse<T>(P.ecx + coarse_packet(agg0, la0, NC, 0), tid - 32, kLoopThreads - 32, np * NC, ep, ecl);
       if (!ok) s_fail = 1;
     }
     __syncthreads();

@@ -369,6 +369,7 @@ struct LoopPart {
   uint32_t* count;            // [nseg] arrivals at barriers
   ulonglong2* ex;             // [kLoopExchanges * kLoopExStride] sums for the leaders
   ulonglong2* line;           // [kLoopLineKinds * kLoopLines] scalars from the leaders
+  // (places: looplayout.h)
   ulonglong2* rcx;            // [3 * pieces] restricted residual
   ulonglong2* ecx;            // [3 * aggregates] coarse correction
   void* pp;                   // [3 * ld] p as packets (8 bytes per value in FP32, 16 in FP64)
