@@ -1219,8 +1219,6 @@ class Engine final : public EngineBase {
   // on these operators (5e-5 of ||b|| at 3M nodes)
   static constexpr double kRtolInner = 1e-4;
 
-  // shared memory of a fused loop (227 KB per block less its static part)
-  static constexpr size_t kLoopSmem = 232448 - 4096;
   // Rows up to which the fused loops run: one mesh, and a batch (whose meshes are groups of blocks
   // that wait only among themselves and stop one by one).  Beyond, a block's vectors outgrow its
   // shared memory and the packets of p, twice the bytes, the L2's share.  ms, fused / separate
@@ -1431,7 +1429,7 @@ class Engine final : public EngineBase {
       a.pinned = pinned_;
       a.shift = !pinned_;
       const int npc = pc ? 1 : 0;
-      a.place = loop_place(epr, 1, npc);
+      a.place = loop_place(B == 1 ? 0 : 1, epr, 1, npc);
       TK(B == 1 ? GSPM_KCLASS_SPMV_MS : GSPM_KCLASS_SPMV_MECH, launch_cg_loop<T>(L_, a, B, 1, npc));
       return GSPM_OK;
     }
@@ -1490,7 +1488,7 @@ class Engine final : public EngineBase {
     if (loop_now()) {
       CgLoop<T> a = loop_args(slot, aval, ld_, x, dinv, 2);
       const int npc = dinv ? 2 : 0;
-      a.place = loop_place(1, nr, npc);
+      a.place = loop_place(2, 1, nr, npc);
       TK(GSPM_KCLASS_SPMV_GS, launch_cg_loop<T>(L_, a, 1, nr, npc));
       return GSPM_OK;
     }
@@ -1557,9 +1555,9 @@ class Engine final : public EngineBase {
   }
 
   // how many of the vectors r, q, p, x, D^-1 fit the shared memory beside the rest
-  int loop_place(int nc, int nr, int pc) const {
+  int loop_place(int kind, int nc, int nr, int pc) const {
     int k = 5;
-    while (k > 0 && loop_smem<T>(nc, nr, pc, k, LP_).total > kLoopSmem) --k;
+    while (k > 0 && loop_smem<T>(nc, nr, pc, k, LP_).total > loop_max_[kind][nr - 1]) --k;
     return k;
   }
 
@@ -1643,9 +1641,14 @@ class Engine final : public EngineBase {
         }
     P.max_ldc[0] = max_ldc[0];
     P.max_ldc[1] = max_ldc[1];
-    for (int nc = 1; nc <= 3; nc += 2)
-      if (loop_smem<T>(nc, 1, pc_ ? 1 : 0, 0, P).total > kLoopSmem) return GSPM_OK;
-    if (loop_smem<T>(1, 3, 2, 0, P).total > kLoopSmem) return GSPM_OK;
+    // (by kind: K^ms, K^mech, GSPM with one to three right-hand sides)
+    for (int kind = 0; kind < 3; ++kind)
+      for (int nr = 1; nr <= (kind == 2 ? 3 : 1); ++nr) {
+        const int pc = kind == 2 ? (dgs_eps_ ? 2 : 0) : (pc_ ? 1 : 0), nc = kind == 1 ? 3 : 1;
+        size_t& most = loop_max_[kind][nr - 1];
+        CK(loop_dynamic_limit<T>(kind, kind == 1 ? 6 : 1, nr, pc, &most));
+        if (loop_smem<T>(nc, nr, pc, 0, P).total > most) return GSPM_OK;
+      }
     auto up = [&](auto** dst, const auto& v) -> int {
       ST(mem_.alloc(dst, (int64_t)v.size()));
       CK(cudaMemcpy(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice));
@@ -2254,6 +2257,7 @@ class Engine final : public EngineBase {
   // fused CG loops
   LoopPart LP_{};
   bool loop_on_ = false;
+  size_t loop_max_[3][3] = {};  // dynamic shared memory by kind and right-hand sides
   // CUDA-graph replay state
   bool graph_on_ = false, capturing_ = false;
   cudaStream_t cap_stream_ = nullptr, body_stream_ = nullptr;

@@ -1002,16 +1002,58 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   }
 }
 
-template <typename T, int B, int NR, int PC, bool KS>
-cudaError_t loop_launch(const Launch& L, const CgLoop<T>& a) {
-  auto k = k_cg_loop<T, B, NR, PC, KS>;
-  const size_t smem = loop_smem<T>(B == 1 ? 1 : 3, NR, PC, a.place, a.part).total;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename T>
+using LoopKernel = void (*)(CgLoop<T>);
+
+// the instantiation of a solve (see launch_cg_loop), or NULL
+template <typename T>
+LoopKernel<T> loop_kernel(int kind, int B, int nr, int pc) {
+  if (B == 6) return pc == 1 ? k_cg_loop<T, 6, 1, 1, true> : k_cg_loop<T, 6, 1, 0, true>;
+  if (B != 1) return nullptr;
+  if (kind != 2) return pc == 1 ? k_cg_loop<T, 1, 1, 1, true> : k_cg_loop<T, 1, 1, 0, true>;
+  switch (pc == 2 ? nr : -nr) {
+    case 1: return k_cg_loop<T, 1, 1, 2, false>;
+    case 2: return k_cg_loop<T, 1, 2, 2, false>;
+    case 3: return k_cg_loop<T, 1, 3, 2, false>;
+    case -1: return k_cg_loop<T, 1, 1, 0, false>;
+    case -2: return k_cg_loop<T, 1, 2, 0, false>;
+    case -3: return k_cg_loop<T, 1, 3, 0, false>;
+  }
+  return nullptr;
+}
+}  // namespace
+
+template <typename T>
+cudaError_t loop_dynamic_limit(int kind, int B, int nr, int pc, size_t* bytes) {
+  *bytes = 0;
+  const LoopKernel<T> k = loop_kernel<T>(kind, B, nr, pc);
+  if (!k) return cudaErrorInvalidValue;
+  int dev = 0, optin = 0, resident = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
   if (e != cudaSuccess) return e;
+  if ((size_t)optin <= fa.sharedSizeBytes) return cudaSuccess;
+  const size_t most = (size_t)optin - fa.sharedSizeBytes;
+  // (one value for every context: a smaller one set by another thread would refuse this one's launch)
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k, kLoopThreads, most);
+  if (e == cudaSuccess && resident > 0) *bytes = most;
+  return e;
+}
+
+template <typename T>
+cudaError_t launch_cg_loop(const Launch& L, const CgLoop<T>& a, int B, int nr, int pc) {
+  (*L.counter) += 1;
+  const LoopKernel<T> k = loop_kernel<T>(a.kind, B, nr, pc);
+  if (!k) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.part.nblocks);
   cfg.blockDim = dim3(kLoopThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = loop_smem<T>(B == 1 ? 1 : 3, nr, pc, a.place, a.part).total;
   cfg.stream = L.stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;  // the blocks wait for one another
@@ -1020,27 +1062,9 @@ cudaError_t loop_launch(const Launch& L, const CgLoop<T>& a) {
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k, a);
 }
-}  // namespace
 
-template <typename T>
-cudaError_t launch_cg_loop(const Launch& L, const CgLoop<T>& a, int B, int nr, int pc) {
-  (*L.counter) += 1;
-  if (B == 6)
-    return pc == 1 ? loop_launch<T, 6, 1, 1, true>(L, a) : loop_launch<T, 6, 1, 0, true>(L, a);
-  if (B != 1) return cudaErrorInvalidValue;
-  if (a.kind != 2)
-    return pc == 1 ? loop_launch<T, 1, 1, 1, true>(L, a) : loop_launch<T, 1, 1, 0, true>(L, a);
-  switch (pc == 2 ? nr : -nr) {
-    case 1: return loop_launch<T, 1, 1, 2, false>(L, a);
-    case 2: return loop_launch<T, 1, 2, 2, false>(L, a);
-    case 3: return loop_launch<T, 1, 3, 2, false>(L, a);
-    case -1: return loop_launch<T, 1, 1, 0, false>(L, a);
-    case -2: return loop_launch<T, 1, 2, 0, false>(L, a);
-    case -3: return loop_launch<T, 1, 3, 0, false>(L, a);
-  }
-  return cudaErrorInvalidValue;
-}
-
+template cudaError_t loop_dynamic_limit<float>(int, int, int, int, size_t*);
+template cudaError_t loop_dynamic_limit<double>(int, int, int, int, size_t*);
 template cudaError_t launch_cg_loop<float>(const Launch&, const CgLoop<float>&, int, int, int);
 template cudaError_t launch_cg_loop<double>(const Launch&, const CgLoop<double>&, int, int, int);
 

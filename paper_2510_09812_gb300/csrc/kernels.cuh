@@ -426,5 +426,10 @@ __host__ __device__ inline LoopSmem loop_smem(int nc, int nr, int pc, int place,
 // 2 Jacobi
 template <typename T>
 cudaError_t launch_cg_loop(const Launch& L, const CgLoop<T>& a, int B, int nr, int pc);
+// Dynamic shared memory that the loop of such a solve can be launched with on the current device: what
+// a block may have less the kernel's static part (up to 4,640 bytes, by instantiation).  0: none.
+// Allows the kernel that much; called before its first launch.
+template <typename T>
+cudaError_t loop_dynamic_limit(int kind, int B, int nr, int pc, size_t* bytes);
 
 }  // namespace gspm
