@@ -449,6 +449,13 @@ GSPM_API int gspm_set_graph(struct gspm_ctx* ctx, int on);
  * again.  Errors: GSPM_ESTATE for host-only contexts. */
 GSPM_API int gspm_set_true_residual(struct gspm_ctx* ctx, int on);
 
+/* Bound of a device-side wait between the blocks of a fused CG loop, in polls (about half a
+ * microsecond each); 0 restores the default of 2^22.  A wait that runs out makes the call return
+ * GSPM_ETIMEOUT: what it had queued behind does no more CG work, the state is not valid, and the
+ * context solves with separate kernels from then on.  In graph mode the next step captures the graph
+ * again.  Errors: GSPM_ESTATE for host-only contexts. */
+GSPM_API int gspm_set_wait_limit(struct gspm_ctx* ctx, uint32_t polls);
+
 /* Change the relative residual targets of the GSPM, K^ms and K^mech solves (gspm_options.rtol_*;
  * Sec. 3.1 uses 1e-7) for the following steps; a value <= 0 keeps that tolerance.  In graph mode
  * the next step captures the graph again.  Errors: GSPM_EINVAL for a tolerance >= 1,

@@ -124,6 +124,7 @@ class EngineBase {
   virtual int set_x0_mode(int mode) = 0;
   virtual int set_graph(int on) = 0;
   virtual int set_true_residual(int on) = 0;
+  virtual int set_wait_limit(uint32_t polls) = 0;
   virtual int set_rtol(double gs, double ms, double mech) = 0;
   virtual int mpnn_params(float* out, const float* in, int64_t count) = 0;
   virtual int mpnn_predict(const double* m, const double* up, const double* up2, double* out,
@@ -546,11 +547,12 @@ class Engine final : public EngineBase {
   }
 
   int check_finite() {
-    ST(check_net());
     CK(cudaMemcpyAsync(host_bad_, bad_, (nseg_ + 1) * sizeof(int), cudaMemcpyDeviceToHost,
                        L_.stream));
     CK(cudaStreamSynchronize(L_.stream));
-    ST(check_loop(host_bad_[nseg_]));
+    const int loop = check_loop(host_bad_[nseg_]);  // (also where the network reports an error)
+    ST(check_net());
+    ST(loop);
     for (int sg = 0; sg < nseg_; ++sg)
       if (host_bad_[sg] > 0) {
         set_error("step: m** not finite or zero at %d magnetic nodes of mesh %d", host_bad_[sg],
@@ -636,6 +638,13 @@ class Engine final : public EngineBase {
   // accumulators and the CG status blocks.
   int set_graph(int on) override {
     graph_on_ = on != 0;
+    return GSPM_OK;
+  }
+
+  // (a captured graph holds the limit)
+  int set_wait_limit(uint32_t polls) override {
+    LP_.polls = polls ? polls : kLoopPolls;
+    ++cfg_gen_;
     return GSPM_OK;
   }
 
@@ -1229,6 +1238,10 @@ class Engine final : public EngineBase {
   // 252,432 14.1 / 17.6, 347,296 16.3 / 20.6, FP64 347,296 56.8 / 68.0, 513,808 29.4 / 27.3.
   static constexpr int64_t kLoopRows = sizeof(T) == 4 ? 400000 : 280000, kLoopBatchRows = 400000;
 
+  // polls of one wait in a fused loop (each is an L2 round trip, well above 0.3 us): seconds, where an
+  // exchange takes microseconds
+  static constexpr uint32_t kLoopPolls = 1u << 22;
+
   template <typename X>
   int upload(T** dst, const std::vector<X>& src) {
     ST(mem_.alloc(dst, (int64_t)src.size()));
@@ -1723,6 +1736,7 @@ class Engine final : public EngineBase {
     CK(cudaMemset(P.ecx, 0, std::max<int64_t>(1, ec) * sizeof(ulonglong2)));
     CK(cudaMemset(P.pp, 0, 3 * ld_ * 2 * sizeof(T)));
     P.err = bad_ + nseg_;
+    P.polls = kLoopPolls;
     LP_ = P;
     ST(stats_alloc());
     loop_on_ = true;
@@ -2596,6 +2610,11 @@ int gspm_set_graph(gspm_ctx* ctx, int on) {
 int gspm_set_true_residual(gspm_ctx* ctx, int on) {
   NEED_ENGINE(ctx);
   return ctx->eng->set_true_residual(on);
+}
+
+int gspm_set_wait_limit(gspm_ctx* ctx, uint32_t polls) {
+  NEED_ENGINE(ctx);
+  return ctx->eng->set_wait_limit(polls);
 }
 
 int gspm_set_rtol(gspm_ctx* ctx, double rtol_gs, double rtol_ms, double rtol_mech) {

@@ -21,7 +21,9 @@
 //    and a barrier (one counter, one polling thread per block: 2400 cycles) a step took 27.0 against
 //    24.8 ms at 198,400 nodes and 54.9 against 51.2 ms at 524,288.
 // A slot is written again only after its readers have answered (argued at each).  Every wait is
-// bounded: a block that gives up sets *err and returns, and so do the others after it.
+// bounded (LoopPart::polls): a block that gives up sets *err and returns, so do the others once their
+// own waits run out, and the loops that are queued behind return at once, until the host has taken
+// the context off the fused loops.
 //
 // Meshes of a batch are independent groups of blocks: they neither wait for one another nor stop
 // together.  Their exchange numbers drift apart, so their packets lie in ranges of their own
@@ -50,9 +52,6 @@ namespace gspm {
 namespace {
 
 constexpr int kNW = kLoopThreads / 32;
-// polls of one wait (each is an L2 round trip, well above 0.3 us): seconds, where an exchange takes
-// microseconds
-constexpr uint32_t kPollLimit = 1u << 22;
 constexpr int kPolls = kLoopMaxBlocks / 32;  // packets per lane
 
 enum { kExPq = 0, kExRr = 1, kExCo = 2 };    // sums to the leader: p.q, of the residual, of servers
@@ -191,12 +190,13 @@ __device__ __forceinline__ void post_sums(ulonglong2* ex, int b, uint32_t ep, co
 
 // Leader, one warp: the sum of the n packets at ex, in *out.  False: gave up.
 template <typename T>
-__device__ __forceinline__ bool sum_posts(const ulonglong2* ex, int n, uint32_t ep, double* out) {
+__device__ __forceinline__ bool sum_posts(const ulonglong2* ex, int n, uint32_t ep, uint32_t polls,
+                                          double* out) {
   const int lane = threadIdx.x & 31;
   ulonglong2 w[kPolls];
   bool ok = false;
 #pragma unroll 1
-  for (uint32_t it = 0; !ok && it < kPollLimit; ++it) {
+  for (uint32_t it = 0; !ok && it < polls; ++it) {
     ok = true;
 #pragma unroll
     for (int u = 0; u < kPolls; ++u)
@@ -225,10 +225,11 @@ __device__ __forceinline__ bool sum_posts(const ulonglong2* ex, int n, uint32_t 
 }
 
 // One warp: payload k of a line into ln[k], k < n.  False: gave up.
-__device__ __forceinline__ bool wait_line(const ulonglong2* line, int k, int n, uint32_t ep, uint2* ln) {
+__device__ __forceinline__ bool wait_line(const ulonglong2* line, int k, int n, uint32_t ep,
+                                          uint32_t polls, uint2* ln) {
   bool ok = k >= n;
 #pragma unroll 1
-  for (uint32_t it = 0; !ok && it < kPollLimit; ++it) {
+  for (uint32_t it = 0; !ok && it < polls; ++it) {
     const ulonglong2 w = ld_pair(line + k);
     ok = fresh(w, ep);
     if (ok) ln[k] = make_uint2((uint32_t)w.x, (uint32_t)w.y);
@@ -237,17 +238,18 @@ __device__ __forceinline__ bool wait_line(const ulonglong2* line, int k, int n, 
   return ok;
 }
 
-// FP32 part of n coarse packets from thread k0 on, every step-th, into dst.  False: gave up.
+// Values of n coarse packets from thread k0 on, every step-th, into dst (FP32: the high words; the low
+// ones are posted as zero).  False: gave up.
 template <typename T>
 __device__ __forceinline__ bool wait_coarse(const ulonglong2* src, int k0, int step, int n, uint32_t ep,
-                                         T* dst) {
+                                            uint32_t polls, T* dst) {
   bool ok = true;
 #pragma unroll 1
-  for (int k = k0; k < n; k += 4 * step) {
+  for (int k = k0; ok && k < n; k += 4 * step) {
     ulonglong2 w[4];
     bool got = false;
 #pragma unroll 1
-    for (uint32_t it = 0; !got && it < kPollLimit; ++it) {
+    for (uint32_t it = 0; !got && it < polls; ++it) {
       got = true;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -320,13 +322,13 @@ struct LineFormat<double, NR, KS> {
 
 // All blocks of the group have published their global stores before any passes: arrivals counted in
 // *count, which reaches `target`.  False: gave up.
-__device__ __forceinline__ bool group_barrier(uint32_t* count, uint32_t target) {
+__device__ __forceinline__ bool group_barrier(uint32_t* count, uint32_t target, uint32_t polls) {
   __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     ok = false;
-    for (uint32_t it = 0; !ok && it < kPollLimit; ++it) {
+    for (uint32_t it = 0; !ok && it < polls; ++it) {
       uint32_t v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
       ok = (int32_t)(v - target) >= 0;
@@ -391,7 +393,7 @@ template <> struct PWord<double> {
 // itself) reads none.  False: gave up.
 template <typename T, int B, int NR, bool DIFF>
 __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ val, int64_t s,
-                                         int lane, const void* pp, uint32_t ep,
+                                         int lane, const void* pp, uint32_t ep, uint32_t polls,
                                          int64_t m_row0, int64_t m_rows,
                                          const T (&xi)[B == 1 ? NR : 3], unsigned skip,
                                          bool valid, T (&acc)[B == 1 ? NR : 3], int k0, int ks) {
@@ -433,7 +435,7 @@ __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ v
         for (int c = 0; c < NV; ++c)
           if (B != 1 || !(skip >> c & 1)) ok &= fresh(x[u][c], ep);
       if (__all_sync(kFull, ok || !valid)) break;
-      if (it >= kPollLimit) return false;
+      if (it >= polls) return false;
     }
     auto get = [&](int u, int c) -> T {
       const T v = PW::val(x[u][c]);
@@ -569,7 +571,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   }
   if (tid == 0) {
     s = a.st[seg];
-    s_fail = 0;
+    s_fail = *(const volatile int*)P.err;
   }
   if (PC == 1) {
     for (int k = tid; k <= np; k += kLoopThreads)
@@ -577,6 +579,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
     for (int k = tid; k < ldc; k += kLoopThreads) rcs[k] = T(0);
   }
   __syncthreads();
+  // a loop before this one gave up: its exchange numbers are not to be met again
+  if (s_fail) return;
   const bool active = s.active;
   const bool proj = KS && s.proj;
   unsigned skip = 0;  // right-hand sides that are done, by value of a row
@@ -640,8 +644,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
         T xi[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) xi[c] = DIFF && row0 + lr < rend ? p.at(c, lr) : T(0);
-        ok = ok && row_part<T, B, NR, DIFF>(a.A, a.val, sl0 + ls, lane, P.pp, ep, m_row0, m_rows, xi,
-                                            skip, row0 + lr < rend, acc, k0, ks);
+        ok = ok && row_part<T, B, NR, DIFF>(a.A, a.val, sl0 + ls, lane, P.pp, ep, P.polls, m_row0,
+                                            m_rows, xi, skip, row0 + lr < rend, acc, k0, ks);
       };
       if (split == 1) {
         for (int ls = warp; ls < nsl; ls += kNW) {
@@ -675,7 +679,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
       if (warp == 0) post_sums<T, NR>(P.ex + kExPq * kLoopExStride, blk, ep, R);
       if (leader) {
         if (warp < NR && !sum_posts<T>(P.ex + kExPq * kLoopExStride + warp * kLoopMaxBlocks + b0, nb,
-                                       ep, tot + warp))
+                                       ep, P.polls, tot + warp))
           s_fail = 1;
         __syncthreads();
         if (warp == 0) {
@@ -698,7 +702,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
         __syncthreads();
         send_lines(P.line + kLnAlpha * kLoopLines + (int64_t)b0 * 8, nb, LF::NA, ep, out);
       }
-      if (warp == 0 && !wait_line(line + kLnAlpha * kLoopLines, lane, LF::NA, ep, ln))
+      if (warp == 0 && !wait_line(line + kLnAlpha * kLoopLines, lane, LF::NA, ep, P.polls, ln))
         s_fail = 1;
       __syncthreads();
       if (s_fail) {
@@ -786,7 +790,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
     if (PC == 1 && g1 > g0) {
       // server: its rows of the dense inverse times the restricted residual; r_c.e_c and the sums of
       // P e_c for the leader
-      if (!wait_coarse<T>(P.rcx + coarse_packet(segp0, segp0, NC, 0), tid, kLoopThreads, segp * NC, ep, pieces))
+      if (!wait_coarse<T>(P.rcx + coarse_packet(segp0, segp0, NC, 0), tid, kLoopThreads, segp * NC, ep,
+                          P.polls, pieces))
         s_fail = 1;
       __syncthreads();
       for (int k = tid; k < nagg * NC; k += kLoopThreads) {
@@ -831,11 +836,11 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
     if (leader) {
       if (warp < VR) {
         if (!sum_posts<T>(P.ex + kExRr * kLoopExStride + warp * kLoopMaxBlocks + b0, nb, ep,
-                          tot + warp))
+                          P.polls, tot + warp))
           s_fail = 1;
       } else if (PC == 1 && warp >= 8 && warp < 9 + NC) {
         if (!sum_posts<T>(P.ex + kExCo * kLoopExStride + (warp - 8) * kLoopMaxBlocks + b0, ns, ep,
-                          totc + warp - 8))
+                          P.polls, totc + warp - 8))
           s_fail = 1;
       }
       __syncthreads();
@@ -899,9 +904,10 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
     {
       bool ok = true;
       if (warp == 0)
-        ok = wait_line(line + kLnBeta * kLoopLines, lane, LF::NB, ep, ln);
+        ok = wait_line(line + kLnBeta * kLoopLines, lane, LF::NB, ep, P.polls, ln);
       else if (PC == 1)
-        ok = wait_coarse<T>(P.ecx + coarse_packet(agg0, la0, NC, 0), tid - 32, kLoopThreads - 32, np * NC, ep, ecl);
+        ok = wait_coarse<T>(P.ecx + coarse_packet(agg0, la0, NC, 0), tid - 32, kLoopThreads - 32, np * NC, ep,
+                            P.polls, ecl);
       if (!ok) s_fail = 1;
     }
     __syncthreads();
@@ -956,7 +962,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
     ulonglong2* slot = P.line + kLnPin * kLoopLines + (int64_t)b0 * 8;
     if (warp == 0) {
       if (blk == pb && lane < NC) post(slot + lane, (double)xval(lane, a.G.seg_pin[seg] - row0), ep);
-      if (!wait_line(slot, lane, NC, ep, ln))
+      if (!wait_line(slot, lane, NC, ep, P.polls, ln))
         s_fail = 1;
     }
     __syncthreads();
@@ -985,7 +991,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   // read their exchange numbers yet.  (Otherwise the leader has heard from every block.)
   if (!active) {
     ++bars;
-    if (!group_barrier(P.count + seg, bars * (uint32_t)nb)) {
+    if (!group_barrier(P.count + seg, bars * (uint32_t)nb, P.polls)) {
       if (tid == 0) atomicExch(P.err, 1);
       return;
     }

@@ -112,6 +112,7 @@ def _load():
         "gspm_set_x0_mode": (C.c_int, [vp, C.c_int]),
         "gspm_set_graph": (C.c_int, [vp, C.c_int]),
         "gspm_set_true_residual": (C.c_int, [vp, C.c_int]),
+        "gspm_set_wait_limit": (C.c_int, [vp, C.c_uint32]),
         "gspm_set_rtol": (C.c_int, [vp, C.c_double, C.c_double, C.c_double]),
         "gspm_coarse_round": (C.c_int, [_dp, C.c_int64, C.c_int, _dp, _dp]),
         "gspm_batch_load": (C.c_int, [C.POINTER(MeshDesc), C.c_int, C.POINTER(Material),
@@ -394,6 +395,11 @@ class Context:
         """Report ||b - K x|| / ||b|| of the last K^ms / K^mech solves in the step stats
         (``gspm_set_true_residual``)."""
         _check(lib.gspm_set_true_residual(self._h, int(bool(on))), "gspm_set_true_residual")
+
+    def set_wait_limit(self, polls: int = 0):
+        """Polls of one device-side wait of a fused CG loop before the call fails with ETIMEOUT
+        (0: the default)."""
+        _check(lib.gspm_set_wait_limit(self._h, int(polls)), "gspm_set_wait_limit")
 
     def set_rtol(self, rtol_gs=0.0, rtol_ms=0.0, rtol_mech=0.0):
         """New CG stopping tolerances for the following steps (<= 0 keeps one)."""
