@@ -1726,15 +1726,16 @@ class Engine final : public EngineBase {
     ST(mem_.alloc(&P.line, ln));
     ST(mem_.alloc(&P.rcx, rc));
     ST(mem_.alloc(&P.ecx, ec));
-    ST(mem_.alloc(&pp, 3 * ld_ * 2 * (int64_t)sizeof(T)));
+    ST(mem_.alloc(&pp, 4 * ld_ * 2 * (int64_t)sizeof(T)));
     P.pp = pp;
+    P.pp1 = pp + 3 * ld_ * 2 * (int64_t)sizeof(T);
     CK(cudaMemset(P.epoch, 0, 2 * S * sizeof(uint32_t)));
     CK(cudaMemset(P.count, 0, S * sizeof(uint32_t)));
     CK(cudaMemset(P.ex, 0, ex * sizeof(ulonglong2)));
     CK(cudaMemset(P.line, 0, ln * sizeof(ulonglong2)));
     CK(cudaMemset(P.rcx, 0, std::max<int64_t>(1, rc) * sizeof(ulonglong2)));
     CK(cudaMemset(P.ecx, 0, std::max<int64_t>(1, ec) * sizeof(ulonglong2)));
-    CK(cudaMemset(P.pp, 0, 3 * ld_ * 2 * sizeof(T)));
+    CK(cudaMemset(P.pp, 0, 4 * ld_ * 2 * sizeof(T)));
     P.err = bad_ + nseg_;
     P.polls = kLoopPolls;
     LP_ = P;

@@ -194,9 +194,8 @@ __device__ __forceinline__ bool sum_posts(const ulonglong2* ex, int n, uint32_t 
                                           double* out) {
   const int lane = threadIdx.x & 31;
   ulonglong2 w[kPolls];
-  bool ok = false;
-#pragma unroll 1
-  for (uint32_t it = 0; !ok && it < polls; ++it) {
+  bool ok;
+  do {
     ok = true;
 #pragma unroll
     for (int u = 0; u < kPolls; ++u)
@@ -204,7 +203,7 @@ __device__ __forceinline__ bool sum_posts(const ulonglong2* ex, int n, uint32_t 
 #pragma unroll
     for (int u = 0; u < kPolls; ++u)
       if (lane + 32 * u < n) ok = ok && fresh(w[u], ep);
-  }
+  } while (!ok && --polls);
   T h = T(0), l = T(0);
 #pragma unroll
   for (int u = 0; u < kPolls; ++u)
@@ -228,10 +227,12 @@ __device__ __forceinline__ bool sum_posts(const ulonglong2* ex, int n, uint32_t 
 __device__ __forceinline__ bool wait_line(const ulonglong2* line, int k, int n, uint32_t ep,
                                           uint32_t polls, uint2* ln) {
   bool ok = k >= n;
-#pragma unroll 1
-  for (uint32_t it = 0; !ok && it < polls; ++it) {
-    const ulonglong2 w = ld_pair(line + k);
-    ok = fresh(w, ep);
+  if (!ok) {
+    ulonglong2 w;
+    do {
+      w = ld_pair(line + k);
+      ok = fresh(w, ep);
+    } while (!ok && --polls);
     if (ok) ln[k] = make_uint2((uint32_t)w.x, (uint32_t)w.y);
   }
   __syncwarp();
@@ -247,9 +248,9 @@ __device__ __forceinline__ bool wait_coarse(const ulonglong2* src, int k0, int s
 #pragma unroll 1
   for (int k = k0; ok && k < n; k += 4 * step) {
     ulonglong2 w[4];
-    bool got = false;
-#pragma unroll 1
-    for (uint32_t it = 0; !got && it < polls; ++it) {
+    bool got;
+    uint32_t left = polls;
+    do {
       got = true;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -257,7 +258,7 @@ __device__ __forceinline__ bool wait_coarse(const ulonglong2* src, int k0, int s
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (k + u * step < n) got = got && fresh(w[u], ep);
-    }
+    } while (!got && --left);
     ok = ok && got;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -327,12 +328,11 @@ __device__ __forceinline__ bool group_barrier(uint32_t* count, uint32_t target, 
   bool ok = true;
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
-    ok = false;
-    for (uint32_t it = 0; !ok && it < polls; ++it) {
+    do {
       uint32_t v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
       ok = (int32_t)(v - target) >= 0;
-    }
+    } while (!ok && --polls);
   }
   return __syncthreads_and(ok);
 }
@@ -388,13 +388,11 @@ template <> struct PWord<double> {
 };
 
 // Part of one SELL row's product with p, neighbours k0, k0 + ks, ...: a round's columns and values
-// are all loaded before its gathers.  p is read as packets of exchange ep (the mesh has m_rows rows
-// from m_row0, see looplayout.h); a lane past the mesh's last row (not valid: its columns point at
-// itself) reads none.  False: gave up.
+// are all loaded before its gathers.  p is read as packets of exchange ep; a lane past the
+// mesh's last row (not valid: its columns point at itself) reads none.  False: gave up.
 template <typename T, int B, int NR, bool DIFF>
 __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ val, int64_t s,
                                          int lane, const void* pp, uint32_t ep, uint32_t polls,
-                                         int64_t m_row0, int64_t m_rows,
                                          const T (&xi)[B == 1 ? NR : 3], unsigned skip,
                                          bool valid, T (&acc)[B == 1 ? NR : 3], int k0, int ks) {
   constexpr int NV = B == 1 ? NR : 3;
@@ -420,13 +418,13 @@ __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ v
       for (int e = 0; e < B; ++e) w[u][e] = __ldcs(bp + e * 32);
     }
     typename PW::W x[U][NV];
-    for (uint32_t it = 0;; ++it) {
+    for (uint32_t left = polls;;) {
       bool ok = true;
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int c = 0; c < NV; ++c) {
-          const int64_t i = B == 1 ? p_packet1(m_row0, m_rows, j[u], c) : p_packet3(j[u], c);
+          const int64_t i = B != 1 ? p_packet3(j[u], c) : (NR == 1 ? p_packet1(j[u]) : p_packet1(j[u], c));
           if (B != 1 || !(skip >> c & 1)) x[u][c] = PW::ld(pp, i);
         }
 #pragma unroll
@@ -435,7 +433,7 @@ __device__ __forceinline__ bool row_part(const DSell& A, const T* __restrict__ v
         for (int c = 0; c < NV; ++c)
           if (B != 1 || !(skip >> c & 1)) ok &= fresh(x[u][c], ep);
       if (__all_sync(kFull, ok || !valid)) break;
-      if (it >= polls) return false;
+      if (!--left) return false;
     }
     auto get = [&](int u, int c) -> T {
       const T v = PW::val(x[u][c]);
@@ -517,7 +515,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   const bool leader = blk == b0;
   const int sl0 = P.sl0[blk], nsl = P.sl1[blk] - sl0;
   const int64_t row0 = (int64_t)sl0 * 32;
-  const int64_t m_row0 = (int64_t)P.sl0[b0] * 32, m_rows = (int64_t)P.sl1[b0 + nb - 1] * 32 - m_row0;
   const int64_t rend = a.G.seg_row0[seg] + a.G.seg_nrow[seg];
   const int64_t pin = a.pinned ? a.G.seg_pin[seg] : -1;
   uint32_t ep = P.epoch[2 * seg], bars = P.epoch[2 * seg + 1];
@@ -545,9 +542,11 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
   const Rows<T, AOS> gp{a.p + gofs, a.ld}, gx{a.x + gofs, a.ld}, gr{a.r + gofs, a.ld};
   const Rows<T, AOS> gd{const_cast<T*>(a.dinv) + gofs, a.ld};
   const Rows<T, AOS> di = PC == 0 ? gd : place(4, const_cast<T*>(a.dinv));
+  void* const pp = B == 1 && NR == 1 ? P.pp1 : P.pp;
   auto publish = [&](int c, int64_t lr, T v) {  // v is row lr's new p
     p.at(c, lr) = v;
-    put_p(P.pp, AOS ? p_packet3(row0 + lr, c) : p_packet1(m_row0, m_rows, row0 + lr, c), v, ep);
+    const int row = (int)(row0 + lr);
+    put_p(pp, AOS ? p_packet3(row, c) : (NR == 1 ? p_packet1(row) : p_packet1(row, c)), v, ep);
   };
   ulonglong2* line = P.line + (int64_t)blk * 8;  // + kLn* * kLoopLines
 
@@ -644,8 +643,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_cg_loop(CgLoop<T> a) {
         T xi[NV];
 #pragma unroll
         for (int c = 0; c < NV; ++c) xi[c] = DIFF && row0 + lr < rend ? p.at(c, lr) : T(0);
-        ok = ok && row_part<T, B, NR, DIFF>(a.A, a.val, sl0 + ls, lane, P.pp, ep, P.polls, m_row0,
-                                            m_rows, xi, skip, row0 + lr < rend, acc, k0, ks);
+        ok = ok && row_part<T, B, NR, DIFF>(a.A, a.val, sl0 + ls, lane, pp, ep, P.polls, xi,
+                                            skip, row0 + lr < rend, acc, k0, ks);
       };
       if (split == 1) {
         for (int ls = warp; ls < nsl; ls += kNW) {

@@ -372,7 +372,7 @@ struct LoopPart {
   // (places: looplayout.h)
   ulonglong2* rcx;            // [3 * pieces] restricted residual
   ulonglong2* ecx;            // [3 * aggregates] coarse correction
-  void* pp;                   // [3 * ld] p as packets (8 bytes per value in FP32, 16 in FP64)
+  void *pp, *pp1;             // [3 * ld], [ld] p as packets (8 bytes per value in FP32, 16 in FP64)
   int* err;                   // set when a wait gave up
   uint32_t polls;             // polls of one wait before it gives up
 };

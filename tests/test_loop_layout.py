@@ -16,9 +16,12 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_2510_09812_gb300", "csrc")
 SRC = """
 #include "looplayout.h"
-extern "C" long p3(long j, int c) { return gspm::p_packet3(j, c); }
-extern "C" long p1(long r0, long rows, long j, int c) { return gspm::p_packet1(r0, rows, j, c); }
-extern "C" long co(long f, long i, int nc, int c) { return gspm::coarse_packet(f, i, nc, c); }
+extern "C" long p3(long j, long c) { return gspm::p_packet3(j, (int)c); }
+extern "C" long q1(long j) { return gspm::p_packet1((int)j); }
+extern "C" long p1(long j, long c) { return gspm::p_packet1((int)j, (int)c); }
+extern "C" long co(long f, long i, long nc, long c) {
+  return gspm::coarse_packet((int)f, (int)i, (int)nc, (int)c);
+}
 """
 
 
@@ -31,9 +34,9 @@ def lay(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(d / "l.so"),
                     str(d / "l.cpp")], check=True)
     lib = C.CDLL(str(d / "l.so"))
-    for f, n in (("p3", 1), ("p1", 3), ("co", 2)):
+    for f, n in (("p3", 2), ("q1", 1), ("p1", 2), ("co", 4)):
         getattr(lib, f).restype = C.c_long
-        getattr(lib, f).argtypes = [C.c_long] * n + [C.c_int] * (2 if f == "co" else 1)
+        getattr(lib, f).argtypes = [C.c_long] * n
     return lib
 
 
@@ -42,8 +45,10 @@ def _solves(lay, first, count, rows):
     items = range(first, first + count)
     if rows:
         yield [lay.p3(j, c) for j in items for c in range(3)]
-        for nr in (1, 2, 3):
-            yield [lay.p1(first, count, j, c) for j in items for c in range(nr)]
+        for nr in (2, 3):
+            yield [lay.p1(j, c) for j in items for c in range(nr)]
+        # one right-hand side: an array of its own
+        yield [-1 - lay.q1(j) for j in items]
     else:
         for nc in (3, 1):
             yield [lay.co(first, i, nc, c) for i in items for c in range(nc)]
@@ -61,7 +66,7 @@ def test_ranges_of_meshes_are_disjoint(lay, counts, rows):
         for solve in _solves(lay, first, count, rows):
             assert len(set(solve)) == len(solve)
             places.update(solve)
-        assert min(places) >= 0 and max(places) < 3 * sum(counts)
+        assert min(places) >= -sum(counts) and max(places) < 3 * sum(counts)
         used.append(places)
     for a, b in itertools.combinations(used, 2):
         assert not a & b
