@@ -38,6 +38,7 @@ def _sources():
         os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "kernels.cuh"),
         os.path.join(CSRC, "device.cuh"),
         os.path.join(CSRC, "flatsum.cuh"), os.path.join(CSRC, "looplayout.h"),
+        os.path.join(CSRC, "sum3.h"),
         os.path.join(CSRC, "mpnn.cuh"),
         os.path.join(INCLUDE, "gspm.h")]
 

@@ -9,10 +9,12 @@
 
 #include <cstdint>
 
+#ifndef GSPM_HD
 #ifdef __CUDACC__
 #define GSPM_HD __host__ __device__
 #else
 #define GSPM_HD
+#endif
 #endif
 
 namespace gspm {
