@@ -937,8 +937,8 @@ class Engine final : public EngineBase {
     }
     // the result goes straight to pinned host memory: no copy after the kernel (45.5 -> 21.3 us a call for
     // 1,024 nodes of three components, of which the flat read is about half)
-    CK(launch_volume_avg(L_, nseg_, avg_max_, avg_node0_, avg_count_, nc, src, w_abi_, host_avg_,
-                         avg_part_, avg_cnt_));
+    CK(launch_volume_avg(L_, nseg_, avg_max_, avg_node0_, avg_count_, avg_part0_, nc, src, w_abi_,
+                         host_avg_, avg_part_, avg_cnt_));
     CK(cudaStreamSynchronize(L_.stream));
     memcpy(out, host_avg_, nseg_ * nc * sizeof(double));
     return GSPM_OK;
@@ -1957,11 +1957,20 @@ class Engine final : public EngineBase {
     ST(mem_.alloc(&w_abi_, nodes_));
     ST(mem_.alloc(&avg_node0_, nseg_));
     ST(mem_.alloc(&avg_count_, nseg_));
-    ST(mem_.alloc(&avg_part_, (int64_t)nseg_ * kSumGrid * kSumComp));
+    // (nine components take the most blocks)
+    std::vector<int64_t> part0(nseg_);
+    int64_t blocks = 0;
+    for (int sg = 0; sg < nseg_; ++sg) {
+      part0[sg] = blocks;
+      blocks += sum_blocks(hb_.seg_nrow[sg], 9);
+    }
+    ST(mem_.alloc(&avg_part0_, nseg_));
+    ST(mem_.alloc(&avg_part_, blocks * kSumComp));
     ST(mem_.alloc(&avg_cnt_, nseg_));
     CK(cudaMemcpy(w_abi_, w.data(), nodes_ * sizeof(double), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(avg_node0_, hb_.seg_node0.data(), nseg_ * 8, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(avg_count_, hb_.seg_nrow.data(), nseg_ * 8, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(avg_part0_, part0.data(), nseg_ * 8, cudaMemcpyHostToDevice));
     CK(cudaMemset(avg_cnt_, 0, nseg_ * sizeof(unsigned)));
     CK(cudaMallocHost(&host_avg_, 9 * (size_t)nseg_ * sizeof(double)));
     avg_max_ = *std::max_element(hb_.seg_nrow.begin(), hb_.seg_nrow.end());
@@ -2267,7 +2276,7 @@ class Engine final : public EngineBase {
   bool pieces_ok_ = false;
   // volume averages in ABI order
   double *w_abi_ = nullptr, *avg_part_ = nullptr, *host_avg_ = nullptr;
-  int64_t *avg_node0_ = nullptr, *avg_count_ = nullptr, avg_max_ = 0;
+  int64_t *avg_node0_ = nullptr, *avg_count_ = nullptr, *avg_part0_ = nullptr, avg_max_ = 0;
   unsigned* avg_cnt_ = nullptr;
   // fused CG loops
   LoopPart LP_{};

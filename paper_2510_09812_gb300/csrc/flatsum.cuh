@@ -3,7 +3,6 @@
 
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <cstdint>
 
 namespace gspm {
@@ -16,10 +15,10 @@ constexpr int64_t kSumOneBlock = 4096;   // values (rows x components) summed by
 
 // Blocks for n rows of nc: up to kSumOneBlock values one block does it all; beyond, a block per round
 // of kSumDeep loads, at most four per SM.
-inline int sum_blocks(int64_t n, int nc) {
+__host__ __device__ inline int sum_blocks(int64_t n, int nc) {
   if (n * nc <= kSumOneBlock) return 1;
-  const int64_t per = (int64_t)kSumDeep * (kSumThreads / nc);
-  return (int)std::min<int64_t>((n + per - 1) / per, kSumGrid);
+  const int64_t per = (int64_t)kSumDeep * (kSumThreads / nc), b = (n + per - 1) / per;
+  return (int)(b < kSumGrid ? b : kSumGrid);
 }
 
 namespace {
@@ -44,7 +43,7 @@ __device__ __forceinline__ double block_sum(double v, int nc, int active, double
   return s;
 }
 
-// out[c] = sum_i w_i f[i*nc + c].  The field is read as the flat array it is: the largest multiple
+// out[c] = sum_i w_i f[i*nc + c], by the blocks blockIdx.x < nblocks.  The field is read as the flat array it is: the largest multiple
 // of nc up to the block size takes part, so a thread keeps one component and one accumulator, and
 // a warp's loads are 256 contiguous bytes (a thread per row reads every 32-byte sector nc times).
 // kSumDeep loads of the field and of the weights are in flight per thread.  The FP64 pipe bounds it
@@ -54,13 +53,13 @@ __device__ __forceinline__ double block_sum(double v, int nc, int active, double
 // (3.5 TB/s; rows of one 133 -> 18 us, of nine 134 -> 66 us).  One block needs neither counter nor
 // scratch and writes `out` itself: 300 rows of three 18.7 -> 4.2 us, against 8.3 us for several
 // blocks and the counter's clear.
-__device__ __forceinline__ void flat_sum(int64_t n, int nc, const double* __restrict__ f,
+__device__ __forceinline__ void flat_sum(int nblocks, int64_t n, int nc, const double* __restrict__ f,
                                          const double* __restrict__ w, double* out,
                                          double* partials, unsigned* counter) {
   __shared__ double sm[kSumThreads];
   __shared__ int last;
   const int rows = kSumThreads / nc, active = rows * nc, t = threadIdx.x;
-  const int64_t step = (int64_t)gridDim.x * rows;
+  const int64_t step = (int64_t)nblocks * rows;
   double v = 0.0;
   if (t < active) {
     int64_t i = (int64_t)blockIdx.x * rows + t / nc;
@@ -79,7 +78,7 @@ __device__ __forceinline__ void flat_sum(int64_t n, int nc, const double* __rest
     }
   }
   double x = block_sum(v, nc, active, sm);
-  if (gridDim.x == 1) {
+  if (nblocks == 1) {
     if (t < nc) out[t] = x;
     return;
   }
@@ -88,18 +87,18 @@ __device__ __forceinline__ void flat_sum(int64_t n, int nc, const double* __rest
     __threadfence();
   }
   __syncthreads();
-  if (t == 0) last = (atomicAdd(counter, 1u) == gridDim.x - 1);
+  if (t == 0) last = (atomicAdd(counter, 1u) == (unsigned)nblocks - 1u);
   __syncthreads();
   if (!last) return;
   __threadfence();
   // the last block to arrive sums the block partials in block order
   v = 0.0;
   if (t < active)
-    for (int b = t / nc; b < (int)gridDim.x; b += kSumDeep * rows) {
+    for (int b = t / nc; b < nblocks; b += kSumDeep * rows) {
       double a[kSumDeep];
 #pragma unroll
       for (int u = 0; u < kSumDeep; ++u)
-        a[u] = b + u * rows < (int)gridDim.x
+        a[u] = b + u * rows < nblocks
                    ? __ldcg(partials + (int64_t)(b + u * rows) * kSumComp + t % nc) : 0.0;
 #pragma unroll
       for (int u = 0; u < kSumDeep; ++u) v += a[u];

@@ -54,17 +54,22 @@ __global__ void __launch_bounds__(kBlock) k_wsum(DSeg G, ItemList IL, int nc, co
   }
 }
 
-// the same for a field in ABI order ([nodes][nc] float64), one grid row per segment
-__global__ void __launch_bounds__(kSumThreads) k_volume_avg(const int64_t* __restrict__ node0,
+// the same for a field in ABI order ([nodes][nc] float64): segments along the grid's rows (as many as it
+// may have, then again), each with the blocks that its own size wants and partials from part0[seg]
+__global__ void __launch_bounds__(kSumThreads) k_volume_avg(int nseg, const int64_t* __restrict__ node0,
                                                             const int64_t* __restrict__ count,
-                                                            int nc, const double* __restrict__ f,
+                                                            const int64_t* __restrict__ part0, int nc,
+                                                            const double* __restrict__ f,
                                                             const double* __restrict__ w,
                                                             double* out, double* partials,
                                                             unsigned* counter) {
-  const int seg = blockIdx.y;
-  const int64_t i0 = node0[seg];
-  flat_sum(count[seg], nc, f + i0 * nc, w + i0, out + seg * nc,
-           partials + (int64_t)seg * kSumGrid * kSumComp, counter + seg);
+  for (int seg = blockIdx.y; seg < nseg; seg += gridDim.y) {
+    const int nb = sum_blocks(count[seg], nc);
+    if ((int)blockIdx.x >= nb) continue;
+    const int64_t i0 = node0[seg];
+    flat_sum(nb, count[seg], nc, f + i0 * nc, w + i0, out + (int64_t)seg * nc,
+             partials + part0[seg] * kSumComp, counter + seg);
+  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -2102,11 +2107,12 @@ cudaError_t launch_wsum(const Launch& L, const DSeg& G, int nc, const T* f, int6
 }
 
 cudaError_t launch_volume_avg(const Launch& L, int nseg, int64_t max_nodes, const int64_t* node0,
-                              const int64_t* count, int nc, const double* f, const double* w,
-                              double* out, double* partials, unsigned* counter) {
+                              const int64_t* count, const int64_t* part0, int nc, const double* f,
+                              const double* w, double* out, double* partials, unsigned* counter) {
   (*L.counter) += 1;
-  k_volume_avg<<<dim3((unsigned)sum_blocks(max_nodes, nc), (unsigned)nseg), kSumThreads, 0,
-                 L.stream>>>(node0, count, nc, f, w, out, partials, counter);
+  const dim3 grid((unsigned)sum_blocks(max_nodes, nc), (unsigned)std::min(nseg, 65535));
+  k_volume_avg<<<grid, kSumThreads, 0, L.stream>>>(nseg, node0, count, part0, nc, f, w, out, partials,
+                                                   counter);
   return cudaGetLastError();
 }
 

@@ -136,11 +136,11 @@ cudaError_t launch_wsum(const Launch& L, const DSeg& G, int nc, const T* f, int6
                         Red red);  // out[seg * nc + c], nc 1, 3 or 6
 // out[seg * nc + c] = sum over segment seg's nodes of w_i f[i * nc + c], f and w in ABI order; segment
 // seg's nodes are count[seg] from node0[seg] (device arrays), max_nodes the largest count.  out may be
-// pinned host memory.  partials: kSumGrid * kSumComp doubles per segment, counter: one per segment,
-// zero between calls (flatsum.cuh).
+// pinned host memory.  partials: kSumComp doubles per block, segment seg's sum_blocks(count[seg], 9)
+// blocks from part0[seg]; counter: one per segment, zero between calls (flatsum.cuh).
 cudaError_t launch_volume_avg(const Launch& L, int nseg, int64_t max_nodes, const int64_t* node0,
-                              const int64_t* count, int nc, const double* f, const double* w,
-                              double* out, double* partials, unsigned* counter);
+                              const int64_t* count, const int64_t* part0, int nc, const double* f,
+                              const double* w, double* out, double* partials, unsigned* counter);
 template <typename T>
 cudaError_t launch_spmv(const Launch& L, const DSell& A, const T* val, int B, const T* x,
                         T* y, int variant = 0, int diff = 0);  // B = 1 scalar, B = 6 or 9 block

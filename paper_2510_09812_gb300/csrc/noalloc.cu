@@ -42,7 +42,7 @@ double* g_addr[kMaxDevices] = {};
 __global__ void __launch_bounds__(gspm::kSumThreads)
 k_wsum_noalloc(int64_t n, int nc, const double* __restrict__ f, const double* __restrict__ w,
                double* __restrict__ out, double* scratch) {
-  gspm::flat_sum(n, nc, f, w, out, scratch,
+  gspm::flat_sum((int)gridDim.x, n, nc, f, w, out, scratch,
                  reinterpret_cast<unsigned*>(scratch + (int64_t)kMaxBlocks * kComp));
 }
 
