@@ -496,8 +496,8 @@ GSPM_API int gspm_mpnn_train(struct gspm_ctx* ctx, int iterations, double lr, ui
 /* ---- measurement ------------------------------------------------------------------------ */
 
 /* kernel classes for gspm_profile_*.  Where a solve's whole CG loop runs as one kernel (meshes up to
- * 400,000 nodes, FP64 280,000, batches 400,000; FP64 at targets up to 1e-10 only), that launch counts
- * as the class of its product. */
+ * 400,000 nodes, FP64 280,000, batches 400,000; FP64 at targets up to 1e-10 only; K^mech only while an
+ * iteration's data fits the L2), that launch counts as the class of its product. */
 #define GSPM_KCLASS_SPMV_MECH 0  /* 3x3-block SpMV + fused p.q of the mechanical CG (K^mech)  */
 #define GSPM_KCLASS_SPMV_GS 1    /* scalar multi-RHS SpMV + p.q of the GSPM CG solves         */
 #define GSPM_KCLASS_SPMV_MS 2    /* scalar SpMV + p.q of the magnetostatic CG (K^ms)          */

@@ -800,7 +800,8 @@ class Engine final : public EngineBase {
     return s;
   }
 
-  // n_steps without a host round trip: graph replays, or direct launches of the fused CG loops;
+  // n_steps without a host round trip: graph replays, or direct launches of the fused CG loops (the
+  // host follows the K^mech loops where those are separate kernels);
   // the statistics come from the device's accumulators and the last step's CG status blocks
   int step_device(int n_steps, const DevParams& D, int printed, gspm_step_stats* st, bool graph) {
     if (graph && (!gexec_ || gexec_x0_ != x0_mode_ || gexec_tres_ != tres_on_ ||
@@ -808,10 +809,14 @@ class Engine final : public EngineBase {
       ST(build_graph(D, printed));
     CK(cudaMemsetAsync(gstats_, 0, 4 * (size_t)nseg_ * sizeof(long long), L_.stream));
     StepInfo si;
-    for (int s = 0; s < n_steps; ++s) {
+    dev_stats_ = !graph;
+    int rc = GSPM_OK;
+    for (int s = 0; s < n_steps && rc == GSPM_OK; ++s) {
       if (graph) CK(cudaGraphLaunch(gexec_, L_.stream));
-      else ST(step_once(D, printed, &si));
+      else rc = step_once(D, printed, &si);
     }
+    dev_stats_ = false;
+    ST(rc);
     if (graph) *L_.counter += graph_static_ * n_steps;
     long long* hst = reinterpret_cast<long long*>(host_graph_);
     unsigned long long* hloops = reinterpret_cast<unsigned long long*>(hst + 4 * nseg_);
@@ -910,7 +915,7 @@ class Engine final : public EngineBase {
     ST(solve_system(kSlotMech, kmech(), kb(), b_, u_, ulo_, rtol, &info));
     TK(GSPM_KCLASS_STRAIN, launch_fstrain<T>(L_, A_, SG_, F_, u_, ulo_, invML_, ebar(), E_, ld));
     if (u) ST(export_field(u_, 1, 3, 3, u, where, ulo_));
-    if (loop_now()) ST(read_mech_info(&info));
+    if (loop_now(kb())) ST(read_mech_info(&info));
     CK(cudaStreamSynchronize(L_.stream));
     int it = 0, nc = 0;
     double rel = 0.0;
@@ -1229,14 +1234,34 @@ class Engine final : public EngineBase {
   static constexpr double kRtolInner = 1e-4;
 
   // Rows up to which the fused loops run: one mesh, and a batch (whose meshes are groups of blocks
-  // that wait only among themselves and stop one by one).  Beyond, a block's vectors outgrow its
-  // shared memory and the packets of p, twice the bytes, the L2's share.  ms, fused / separate
-  // kernels: two mixed steps at 66,816 nodes 13.3 / 25.1, 198,400 24.0 / 34.2, 300,000 29.1 / 35.2,
-  // 396,000 39.5 / 42.0, 449,280 55.9 / 44.6, 524,288 50.2 / 48.8; FP64 100,800 45.9 / 58.9, 198,400
-  // 77.4 / 84.8, 300,000 103.4 / 104.0, 396,000 147.7 / 132.8; elastic solves 152,969 6.9 / 9.3,
-  // 300,000 11.5 / 12.2, 396,000 16.0 / 14.4, FP64 300,000 33.6 / 30.6; batches 82,064 7.3 / 12.0,
-  // 252,432 14.1 / 17.6, 347,296 16.3 / 20.6, FP64 347,296 56.8 / 68.0, 513,808 29.4 / 27.3.
+  // that wait only among themselves and stop one by one).  ms, fused / separate kernels: two mixed
+  // steps at 163,840 nodes 22.8 / 32.5, 296,000 29.8 / 36.5, 336,000 34.2 / 38.8, 400,000 40.1 / 42.0,
+  // 495,000 56.7 / 46.1; FP64 131,072 55.4 / 85.6, 204,800 80.6 / 104.8, 276,480 105.6 / 123.9; batches
+  // 92,160 16.4 / 25.1, 276,480 27.8 / 36.8, 368,640 32.6 / 38.3, FP64 276,480 91.0 / 111.0.
   static constexpr int64_t kLoopRows = sizeof(T) == 4 ? 400000 : 280000, kLoopBatchRows = 400000;
+
+  // Whether the K^mech solves take the fused loop too: what an iteration streams should stay in the L2
+  // (129 MB).  That is x, the values and columns of K^mech and the packets of p, and y, the coarse inverse,
+  // which the loop reads whole where the separate kernels read its triangle.  Elastic solves, us per
+  // iteration, fused / separate (MB of x + y): mixed 65,536 nodes 23.0 / 38.5 (29 + 0.3), 31.1 / 42.6
+  // (29 + 19), 48.2 / 51.3 (29 + 72); 163,840 42.6 / 49.2 (73 + 2), 52.3 / 53.9 (73 + 28), 62.0 / 56.9
+  // (73 + 50), 100.7 / 63.3 (73 + 118); 256,000 54.0 / 57.8 (114 + 5), 64.1 / 62.1 (114 + 31), 81.7 / 68.4
+  // (114 + 78); 296,000 58.2 / 59.7 (132 + 8); 336,000 65.5 / 62.3 (150 + 8), 150.7 / 75.4 (150 + 118);
+  // 400,000 77.2 / 70.5 (178 + 11).  FP64, where the arithmetic hides more of it: 65,536 88.9 / 114.6
+  // (54 + 75), 163,840 166.3 / 166.5 (136 + 112), 256,000 151.1 / 157.3 (212 + 17), 189.8 / 179.7
+  // (212 + 78), 276,480 165.2 / 168.6 (229 + 23), 320,000 188.6 / 187.6 (265 + 26).  Batches gain more
+  // (each mesh stops by itself): mixed solves, ms, 368,640 nodes 11.8 / 12.2 (164), 460,800 14.6 / 16.7.
+  // With K^mech separate and the scalar solves fused two mixed steps take 33.8 ms at 336,000 nodes
+  // (34.2 all fused), 38.0 at 400,000 (40.1).
+  bool loop_mech_pays() const {
+    const double w = sizeof(T);
+    const double x = (6 * w + 4) * (double)entries_ + 6 * w * (double)n_;
+    double y = 0.0;
+    for (const HostCoarse& c : hb_.coarse)
+      y += 9.0 * (double)c.n_agg * (double)c.n_agg * sizeof(typename CoarseStore<T>::type);
+    if (sizeof(T) == 8) return x + y <= 255e6;
+    return x + 1.5 * y <= (nseg_ == 1 ? 140e6 : 200e6);
+  }
 
   // polls of one wait in a fused loop (each is an L2 round trip, well above 0.3 us): seconds, where an
   // exchange takes microseconds
@@ -1355,7 +1380,8 @@ class Engine final : public EngineBase {
   static constexpr double kFastRtol = 1e-10;
   static constexpr bool kRounded = sizeof(T) == 4;
   void set_fast(double rtol) { fast_ = kRounded || rtol <= kFastRtol; }
-  bool loop_now() const { return loop_on_ && fast_; }
+  bool loop_now() const { return loop_on_ && fast_; }                    // K^ms and GSPM solves
+  bool loop_now(int B) const { return loop_now() && (B == 1 || loop_mech_); }
   const T* kmech() const { return !fast_ && Kmech9_ ? Kmech9_ : Kmech_; }
   int kb() const { return !fast_ && Kmech9_ ? 9 : kb_; }
   int var_block() const { return !fast_ && Kmech9_ ? var_block9_ : var_block_; }
@@ -1383,7 +1409,7 @@ class Engine final : public EngineBase {
       CK(cudaMemsetAsync(dx_, 0, len * sizeof(T), L_.stream));
       ST(solve_general(slot2, val, B, b, x, dx_, rtol, &i2));
       TK(GSPM_KCLASS_CG_INIT, launch_refine_add<T>(L_, len, x, xlo, dx_));
-      if (!capturing_ && !loop_now()) {
+      if (!capturing_ && !loop_now(B)) {
         info->assign(nseg_, SolveInfo());
         for (int sg = 0; sg < nseg_; ++sg) {
           (*info)[sg].iters = i1[sg].iters + i2[sg].iters;
@@ -1436,7 +1462,7 @@ class Engine final : public EngineBase {
       return GSPM_OK;
     };
     TK(GSPM_KCLASS_CG_INIT, launch_cg_init<T>(L_, A_, SG_, val, B, b, x0, r_, p_, st, na, rtol, opt_.max_iter, red_, pinned_ ? nullptr : bmean, pinned_, pc ? 1 : 0));
-    if (loop_now()) {
+    if (loop_now(B)) {
       if (!pinned_ && !pc) TK(GSPM_KCLASS_CG_INIT, launch_cg_psub<T>(L_, A_, SG_, epr, p_, st));
       CgLoop<T> a = loop_args(slot, val, len, x, dinv, B == 1 ? 0 : 1);
       a.pinned = pinned_;
@@ -1482,6 +1508,7 @@ class Engine final : public EngineBase {
       ST(cg_graph_loop(slot, iter, B == 1 ? 0 : 1, runs ? 6 : (pc ? 7 : 3)));
     else
       ST(cg_loop(slot, iter, info));
+    if (!capturing_ && dev_stats_) CK(launch_solve_stats(L_, st, nseg_, B == 1 ? 0 : 1, gstats_));
     // singular system: move the solution to the pinned one (zero at the pinned node)
     if (!pinned_) TK(GSPM_KCLASS_CG_INIT, launch_pin_shift<T>(L_, A_, SG_, epr, x, xpin));
     TK(GSPM_KCLASS_CG_INIT, launch_cg_zero<T>(L_, SG_, epr, x, st));
@@ -1575,17 +1602,18 @@ class Engine final : public EngineBase {
   }
 
   // Rows to blocks for the fused loops, or loop_on_ = false where they do not apply: aggregates
-  // that are not runs of rows, more meshes than blocks, operators without symmetric blocks, or
-  // a size at which the separate kernels are as fast (see kLoopRows).
+  // that are not runs of rows, more meshes than blocks, or a size at which the separate kernels are
+  // as fast (see kLoopRows).  loop_mech_ = false: only the scalar solves (K^mech without symmetric
+  // blocks, or see loop_mech_pays).
   int init_loop() {
     const int S = nseg_;
     const int max_blocks = std::min(L_.sms, kLoopMaxBlocks);
     int coop = 0, dev = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-    if (!coop || kb_ != 6 || S > max_blocks || n_ > (S == 1 ? kLoopRows : kLoopBatchRows))
-      return GSPM_OK;
+    if (!coop || S > max_blocks || n_ > (S == 1 ? kLoopRows : kLoopBatchRows)) return GSPM_OK;
     if (pc_ && !CC_.contig) return GSPM_OK;
+    bool mech = kb_ == 6 && loop_mech_pays();
     // blocks per mesh: one each, the rest to whichever mesh has the most slices per block
     std::vector<int64_t> nb(S, 1);
     for (int left = max_blocks - S; left > 0; --left) {
@@ -1660,7 +1688,9 @@ class Engine final : public EngineBase {
         const int pc = kind == 2 ? (dgs_eps_ ? 2 : 0) : (pc_ ? 1 : 0), nc = kind == 1 ? 3 : 1;
         size_t& most = loop_max_[kind][nr - 1];
         CK(loop_dynamic_limit<T>(kind, kind == 1 ? 6 : 1, nr, pc, &most));
-        if (loop_smem<T>(nc, nr, pc, 0, P).total > most) return GSPM_OK;
+        if (loop_smem<T>(nc, nr, pc, 0, P).total <= most) continue;
+        if (kind != 1) return GSPM_OK;
+        mech = false;
       }
     auto up = [&](auto** dst, const auto& v) -> int {
       ST(mem_.alloc(dst, (int64_t)v.size()));
@@ -1687,7 +1717,7 @@ class Engine final : public EngineBase {
       P.pc0 = d_pc0;
       P.ap = d_ap;
       P.pc_row = d_prow;
-      for (int e = 0; e < 2; ++e) {
+      for (int e = mech ? 0 : 1; e < 2; ++e) {
         std::vector<int64_t> off(S);
         std::vector<int32_t> ldv(S);
         int64_t total = 0;
@@ -1741,6 +1771,7 @@ class Engine final : public EngineBase {
     LP_ = P;
     ST(stats_alloc());
     loop_on_ = true;
+    loop_mech_ = mech;
     return GSPM_OK;
   }
 
@@ -2280,7 +2311,8 @@ class Engine final : public EngineBase {
   unsigned* avg_cnt_ = nullptr;
   // fused CG loops
   LoopPart LP_{};
-  bool loop_on_ = false;
+  bool loop_on_ = false, loop_mech_ = false;  // K^ms and GSPM solves; K^mech too
+  bool dev_stats_ = false;  // separate loops add to gstats_
   size_t loop_max_[3][3] = {};  // dynamic shared memory by kind and right-hand sides
   // CUDA-graph replay state
   bool graph_on_ = false, capturing_ = false;
