@@ -658,6 +658,19 @@ def run_dt_sweep(args):
 # the headline
 # ------------------------------------------------------------------------------------------
 
+def kernel_row(desc, nbytes, t_ms, launches, peak, products=None):
+    """Time and bandwidth of a kernel class from its profiled launches.  products: how many matrix
+    products the pass did, for a class whose launch may be a whole CG loop (then there are fewer
+    launches): such a launch does more than a product's bytes, so it has a time but no bandwidth."""
+    loop = products is not None and 0 < launches < products
+    gbs = nbytes * launches / (t_ms / 1000.0) / 1e9 if t_ms > 0 and not loop else None
+    return {"kernel": "k_cg_loop (whole CG loops, %.1f products each)" % (products / launches)
+            if loop else desc,
+            "bytes_per_launch": None if loop else int(nbytes), "launches": launches,
+            "us_per_launch": 1000.0 * t_ms / launches if launches else None,
+            "achieved_gbs": gbs, "frac": gbs / peak if gbs else None}
+
+
 def run_ours(args):
     import torch
     ws, rank, local = _dist()
@@ -758,9 +771,10 @@ def run_ours(args):
     # kernel pass (separate, from the same state): CUDA events around every launch of the
     # mechanical SpMV and of the four assembly / recovery row kernels
     w = 4 if precision == "mixed" else 8
+    blk = 6 if precision == "mixed" else 9   # values per block (FP64 at 1e-7: see gspm_options.rtol_gs)
     E, S = info["sell_entries"], (n + 31) // 32
     kern = {  # algorithmic bytes per launch: values + columns + slice headers + vectors
-        "spmv_mech": ("k_cg_spmv<B=6> (symmetric 3x3-block SELL SpMV + p.q)", E * (6 * w + 4) + S * 12 + 6 * n * w),
+        "spmv_mech": (f"k_cg_spmv<B={blk}> (3x3-block SELL SpMV + p.q)", E * (blk * w + 4) + S * 12 + 6 * n * w),
         "rhs_ms": ("k_fdiv (b^ms = F^ms m)", E * (3 * w + 4) + S * 12 + 3 * n * w + n * w),
         "grad_ms": ("k_fgrad (h~_d = -grad U)", E * (3 * w + 4) + S * 12 + n * w + 8 * n + 3 * n * w),
         "rhs_mech": ("k_gdiv (b^mech = F^mech E0)", E * (3 * w + 4) + S * 12 + 6 * n * w + 3 * n * w),
@@ -771,12 +785,9 @@ def run_ours(args):
     _, st_k, _, prof, _ = timed(ctx, kp, tuple(kern))
     rooflines = {}
     for c, (desc, nbytes) in kern.items():
-        t_ms, cnt = prof[c]
-        gbs = nbytes * cnt / (t_ms / 1000.0) / 1e9 if t_ms > 0 else None
-        rooflines[c] = {"kernel": desc, "bytes_per_launch": int(nbytes), "launches": cnt,
-                        "us_per_launch": 1000.0 * t_ms / cnt if cnt else None,
-                        "achieved_gbs": gbs, "frac": gbs / peak if gbs else None,
-                        "traffic": _traffic(c) if args.cells is None else None}
+        rooflines[c] = kernel_row(desc, nbytes, *prof[c], peak,
+                                  st_k["it_mech"] if c == "spmv_mech" else None)
+        rooflines[c]["traffic"] = _traffic(c) if args.cells is None else None
     sp = rooflines["spmv_mech"]
     roofline = {"bound": "hbm", "kernel": sp["kernel"], "achieved": sp["achieved_gbs"],
                 "peak": peak, "unit": "GB/s", "frac": sp["frac"], "traffic": sp["traffic"],
