@@ -29,16 +29,29 @@
 // together.  Their exchange numbers drift apart, so their packets lie in ranges of their own
 // (looplayout.h; ex and line are per block).
 //
-// Measured (separate kernels -> fused): time steps at 1,024 nodes (FP64) 7.8 -> 3.1 ms, 19,305 nodes
-// (mixed) 14.8 -> 5.8, 65,536 (mixed) 18.4 -> 7.0, 65,536 hexahedra (FP64) 22.6 -> 12.6; an elastic
-// solve at 152,969 nodes 13.9 -> 7.4 ms; larger sizes at kLoopRows.  An iteration of K^mech at
-// 19,305 nodes takes 43,000 cycles: 5,000 for the product, 2,500 for the vectors, the rest the chain
-// of exchanges (two hops for p.q, three for the residual and the coarse correction, one for p).  What
-// bounds it is that chain of dependent hops and single-warp sums, not bandwidth; at 65,536 hexahedra
-// in FP64 half of it is the FP64 pipe (27 x 9 multiply-adds per row at two per clock and SM).
-// Tried and slower: clusters of 4 to 16 blocks with the sums in distributed shared memory (12.4 to
-// 14.7 ms for the first figure's 12.4, 29.7 for the third's 21.0: fewer SMs hold clusters), helper
-// functions out of line, and warps waiting by nanosleep instead of at the barrier.
+// Measured, separate kernels -> fused: three mixed steps at 19,305 nodes 44.0 -> 16.4 ms, at 65,536
+// 56.4 -> 20.4; two FP64 steps at 65,536 hexahedra 44.9 -> 25.0; an elastic solve at 152,969 nodes
+// 14.9 -> 7.2 ms; larger sizes at kLoopRows.  Cycles of a K^mech iteration (clock64 in the leader's and a
+// server's first thread, mean of a solve):
+//                            19,305 mixed   65,536 mixed   152,969 mixed   65,536 hexahedra FP64
+//   product                        6,650         13,700          31,700          86,400
+//   p.q at the leader, summed      6,200          7,100           8,400          11,300
+//   alpha, lines to the blocks     3,350          3,400           3,150           3,750
+//   vectors, pieces                3,430          3,750           6,650          16,100
+//   server: pieces arrive          3,700          3,850           4,050           5,100
+//     gather, inverse x pieces     8,800          5,050           5,200           6,300
+//   leader: sums arrive            4,350          6,200           4,800           5,500
+//     decisions                    2,600          3,050           3,100           2,800
+//   beta, correction received      2,350          1,600           2,400           2,700
+//   p                                900          1,300           2,700           2,900
+// (a hop between two SMs is 1,400).  So up to 65,536 nodes the serial sections of the leader and the
+// servers and the hops between them bound it, not bandwidth; in FP64 the product does, by the FP64 pipe
+// (27 x 9 multiply-adds per row at two per clock and SM).  The kernels spill (128 registers per thread at
+// 512 threads: 596 bytes loaded in the mixed K^mech loop, 380 in FP64, none in the plain scalar ones).
+// Tried, no faster: clusters of 4 to 16 blocks with the sums in distributed shared memory (12.4 to
+// 14.7 ms for four FP64 steps at 1,024 nodes that took 12.4 without, 29.7 for three mixed ones at 65,536
+// that took 21.0: fewer SMs hold clusters), helper functions out of line, and warps waiting by
+// nanosleep instead of at the barrier.
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -43,16 +43,16 @@ __device__ __forceinline__ double block_sum(double v, int nc, int active, double
   return s;
 }
 
-// out[c] = sum_i w_i f[i*nc + c], by the blocks blockIdx.x < nblocks.  The field is read as the flat array it is: the largest multiple
-// of nc up to the block size takes part, so a thread keeps one component and one accumulator, and
-// a warp's loads are 256 contiguous bytes (a thread per row reads every 32-byte sector nc times).
-// kSumDeep loads of the field and of the weights are in flight per thread.  The FP64 pipe bounds it
-// (two FMAs per SM and clock: 30 us for 3M rows of six, against 25 us for the bytes), so the
-// reduction trees must stay small against the rows: four blocks per SM and no more.  At 2,963,088
-// rows of six: 136.1 us before (thread per row, 2048 blocks, nine warp trees each), 47.2 us now
-// (3.5 TB/s; rows of one 133 -> 18 us, of nine 134 -> 66 us).  One block needs neither counter nor
-// scratch and writes `out` itself: 300 rows of three 18.7 -> 4.2 us, against 8.3 us for several
-// blocks and the counter's clear.
+// out[c] = sum_i w_i f[i*nc + c], by the blocks blockIdx.x < nblocks.  The field is read as the flat
+// array it is: the largest multiple of nc up to the block size takes part, so a thread keeps one
+// component and one accumulator, and a warp's loads are 256 contiguous bytes (a thread per row reads
+// every 32-byte sector nc times).  kSumDeep loads of the field and of the weights are in flight per
+// thread.  The FP64 pipe bounds it (two FMAs per SM and clock: 28 us for 3M rows of six, against 25 us
+// for the bytes), so the reduction trees must stay small against the rows: four blocks per SM and no
+// more.  At 2,963,088 rows of six: 136.1 us before (thread per row, 2048 blocks, nine warp trees each),
+// 47.2 us now with the counter's clear, a launch of its own (3.5 TB/s; rows of one 133 -> 18 us, of nine
+// 134 -> 66 us).  One block needs neither counter nor scratch and writes `out` itself: 300 rows of three
+// 18.7 -> 4.2 us, against 8.3 us for several blocks and the counter's clear.
 __device__ __forceinline__ void flat_sum(int nblocks, int64_t n, int nc, const double* __restrict__ f,
                                          const double* __restrict__ w, double* out,
                                          double* partials, unsigned* counter) {
