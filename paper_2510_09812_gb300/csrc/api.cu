@@ -1373,8 +1373,8 @@ class Engine final : public EngineBase {
   // Two CG runs on one system whose sums differ in rounding only agree within a good part of their
   // stopping tolerance, not within rounding: orthogonality is lost on the way, and a residual near
   // the tolerance may end a run one iteration earlier.  FP64 solutions (2-norm, relative) of the fused
-  // loops against the separate kernels: up to 2.8e-8 at 1e-7, 5.9e-9 at 1e-8, 1.0e-9 at 1e-9, 5e-11 at
-  // 1e-10.  So an FP64 call whose solves stop above kFastRtol keeps one arithmetic at every size: the
+  // loops against the separate kernels: up to 2.8e-8 at 1e-7, 5.9e-9 at 1e-8, 1.0e-9 at 1e-9, 1.8e-10
+  // at 1e-10.  So an FP64 call whose solves stop above kFastRtol keeps one arithmetic at every size: the
   // separate kernels with z stored, nine values per block and the sums of seg_reduce_fixed.  Tighter
   // ones, and all of mixed precision (whose results are held in FP32), take the fast forms.
   static constexpr double kFastRtol = 1e-10;
@@ -1687,7 +1687,10 @@ class Engine final : public EngineBase {
       for (int nr = 1; nr <= (kind == 2 ? 3 : 1); ++nr) {
         const int pc = kind == 2 ? (dgs_eps_ ? 2 : 0) : (pc_ ? 1 : 0), nc = kind == 1 ? 3 : 1;
         size_t& most = loop_max_[kind][nr - 1];
-        CK(loop_dynamic_limit<T>(kind, kind == 1 ? 6 : 1, nr, pc, &most));
+        if (loop_dynamic_limit<T>(kind, kind == 1 ? 6 : 1, nr, pc, &most) != cudaSuccess) {
+          cudaGetLastError();  // (not this context's to report: it solves with separate kernels)
+          return GSPM_OK;
+        }
         if (loop_smem<T>(nc, nr, pc, 0, P).total <= most) continue;
         if (kind != 1) return GSPM_OK;
         mech = false;
